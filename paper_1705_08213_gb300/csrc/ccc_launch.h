@@ -106,6 +106,9 @@ struct Tally2Args {
   float threshold = 0.f;
   // Column blocks per L2 group of the tensor-core tile order (0 = default 8).
   int32_t group = 0;
+  // Cycles between the output lines of a tile in the SM-pair kernels (set by
+  // their launches; 0 = stored as fast as they come).
+  uint32_t pace = 0;
   // Row range of a phase: only pairs with i_begin <= i < i_end are computed and
   // pair (i, j) is stored at index pair_index(i, j) - pair0.
   int64_t i_begin = 0;

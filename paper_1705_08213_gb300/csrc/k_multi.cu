@@ -270,7 +270,7 @@ __global__ void k_metric2_multi(const int32_t *__restrict__ tally, const float *
       continue;
     }
     const float d = static_cast<float>(n4);
-    const float inv = __frcp_rn(d);
+    const float inv = rcp_count(d);
     for (int a = 0; a < s; ++a) {
       float wi;
       if (norm == CCC_NORM_PERSNP) {
@@ -278,7 +278,7 @@ __global__ void k_metric2_multi(const int32_t *__restrict__ tally, const float *
       } else {
         int32_t rs = 0;
         for (int b = 0; b < s; ++b) rs += t[a * s + b];
-        wi = joint_factor(rs, d, gamma);
+        wi = joint_factor(static_cast<float>(rs), d, inv, gamma);
       }
       for (int b = 0; b < s; ++b) {
         const float r = static_cast<float>(t[a * s + b]);
@@ -287,7 +287,8 @@ __global__ void k_metric2_multi(const int32_t *__restrict__ tally, const float *
         } else {
           int32_t cs = 0;
           for (int x = 0; x < s; ++x) cs += t[x * s + b];
-          out[a * s + b] = __fmul_rn(__fmul_rn(__fdiv_rn(r, d), wi), joint_factor(cs, d, gamma));
+          out[a * s + b] = __fmul_rn(__fmul_rn(div_count(r, d, inv), wi),
+                                     joint_factor(static_cast<float>(cs), d, inv, gamma));
         }
       }
     }

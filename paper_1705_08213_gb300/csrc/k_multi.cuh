@@ -83,10 +83,14 @@ struct EpiMultiT {
 
   // The warps of column half h (c0 = h NC) take the chunks of 32 columns
   // [h NBQ / 2, (h + 1) NBQ / 2); chunk c is B quarter NBQ J + c.
+  template <int NC>
+  __device__ __forceinline__ static tcp::NoEarly early(const Params &, const Sched &, int, int, int, int) {
+    return {};
+  }
   template <int NC, bool PRELOAD = false>
   __device__ static void tile(const Params &args, const Sched &sc, int rank, int quarter,
                               int lane, uint32_t t_base, uint32_t release_cluster_bar, int c0,
-                              float *stage) {
+                              float *stage, tcp::NoEarly, bool) {
     static_assert(!PRELOAD, "s-state tiles run on the two-accumulator pipeline");
     static_assert(NBQ % 2 == 0, "two column halves");
     const int cb = (c0 / NC) * (NBQ / 2);
@@ -153,22 +157,19 @@ struct EpiMultiT {
         store_row<S>(args.tally + base, r);
         if (!want_ccc) continue;
         float cv[S];
-        if (n4 == 0) {
-#pragma unroll
-          for (int b = 0; b < S; ++b) cv[b] = 0.f;
-        } else if (persnp) {
-          const float inv = __frcp_rn(static_cast<float>(n4));
+        const float d = n4 == 0 ? 1.f : static_cast<float>(n4);
+        const float inv = rcp_count(d);
+        if (persnp) {
           const float *wjs = stage + ((c - cb) * PW + jl) * S;
 #pragma unroll
           for (int b = 0; b < S; ++b)
             cv[b] = __fmul_rn(__fmul_rn(__fmul_rn(static_cast<float>(r[b]), inv), wi), wjs[b]);
         } else {
-          const float d = static_cast<float>(n4);
-          const float wia = joint_factor(rs, d, args.gamma);
+          const float wia = joint_factor(static_cast<float>(rs), d, inv, args.gamma);
 #pragma unroll
           for (int b = 0; b < S; ++b) {
-            const float wjb = joint_factor(colsum[b], d, args.gamma);
-            cv[b] = __fmul_rn(__fmul_rn(__fdiv_rn(static_cast<float>(r[b]), d), wia), wjb);
+            const float wjb = joint_factor(static_cast<float>(colsum[b]), d, inv, args.gamma);
+            cv[b] = __fmul_rn(__fmul_rn(div_count(static_cast<float>(r[b]), d, inv), wia), wjb);
           }
         }
         store_row<S>(args.ccc + base, cv);
@@ -185,10 +186,14 @@ struct EpiMultiSplit {
   static constexpr int PW = snps_per_quarter(S);
   static constexpr int STAGE_BYTES_PER_WARP = 0;
 
+  template <int NC>
+  __device__ __forceinline__ static tcp::NoEarly early(const Params &, const SplitSchedPair &, int, int, int, int) {
+    return {};
+  }
   template <int NC, bool PRELOAD = false>
   __device__ static void tile(const Params &args, const SplitSchedPair &sc, int rank, int quarter,
                               int lane, uint32_t t_base, uint32_t release_cluster_bar, int c0,
-                              float *) {
+                              float *, tcp::NoEarly, bool) {
     static_assert(!PRELOAD, "s-state tiles run on the two-accumulator pipeline");
     const int u = lane / S;
     const int a = lane - u * S;

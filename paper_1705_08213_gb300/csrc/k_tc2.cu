@@ -163,109 +163,251 @@ struct Epi2 {
   }
 };
 
-// SM-pair epilogue with the chunk staged in shared memory.  Lane (2i + a)
-// holds row (i, a) of a 32 x 32 accumulator chunk (16 SNPs i x 16 SNPs j);
-// written row by row to `stage` (stride 33 floats, no bank conflicts), it is
-// read back so that in store t lanes 0-15 and 16-31 each take 16 consecutive
-// j of one SNP i: every warp store then covers two 256-byte runs of the
-// output instead of sixteen 32-byte ones (GB300, 20,000 x 16,384: 6.32 against
-// 6.37 ms per launch; thresholded output, which stores few pairs, keeps the
-// unstaged body: staging made it 5% slower).
+// SM-pair epilogue of full output.  Lane (2i + a) of a warp holds row (i, a) of
+// the accumulator, 16 SNPs i by JW SNPs j.  Eight j at a time, the warp writes
+// its rows into a ring of two 8-j pieces in shared memory, laid out as whole
+// 2 x 2 tables (16 bytes), and reads back, for each SNP i, the eight tables
+// that fill one 128-byte line of the output: lane 8 g + l of store t takes SNP
+// i = 4 t + g and table l of the line.  The triangle's rows start at any
+// multiple of 16 bytes, so a line lies across two pieces by the row's own
+// offset; every warp store covers four whole lines, but for each row's first
+// and last.
+//
+// What bounds it: an SM's stores and its operand loads share the way to L2, so
+// the stores are made in as few packets as possible (four lines per warp store;
+// two 256-byte runs at any offset took six), and spread over the tile (pace()).
+// Stores alone, 20,000 SNPs, 6.4 GB: 1.19 ms as here, 1.36 ms as 256-byte runs.
+// The two epilogue warps of a scheduler have nothing to hide latency behind
+// but their own independent iterations, so an iteration is short (about 35
+// instructions, against 119 with conversions, IEEE divisions with their
+// branches and a 64-bit index per pair) and free of branches: the float
+// accumulators are used as they are, and pairs that are not stored (i >= j,
+// past n_v, outside the phase) only predicate the stores.
+// Per call (GB300), before -> now: 20,000 SNPs x 4,096 2.13 -> 1.60 ms (4.0 TB/s),
+// x 16,384 3.74 -> 3.62 ms; 3,001 x 2,503 JOINT 92 -> 46 us.
 struct Epi2Staged {
-  static constexpr int STRIDE = 33;
-  static constexpr int STAGE_BYTES_PER_WARP = 32 * STRIDE * 4;
+  static constexpr int STAGE_BYTES_PER_WARP = 16 * 256;  // 16 SNPs i x 16 tables
+  static constexpr int RING_BYTES_PER_WARP = 16 * 8;     // the factors w_j of the ring's 16 j
+  static constexpr size_t extra_bytes(int ew) { return static_cast<size_t>(ew) * RING_BYTES_PER_WARP; }
+
+  enum Mode { TALLY, PERSNP, JOINT };
+
+  // Cycles from line to line that spread a tile's lines (2 NC + 1, NC = 32 / ew
+  // chunks per warp) over about 4/5 of the MMAs of the next tile, K stages of
+  // about 640 (e2m1) or 560 (e4m3) cycles; kLineCycles is what a line's stores
+  // take by themselves.  20,000 SNPs, all panels' tiles in lockstep: stored as
+  // they come, the burst of each tile's 512 KB delays the operand loads
+  // (16,384 individuals 3.89 ms, 8,192 2.45 ms, 4,096 1.67 ms); spread, and the
+  // warps one after another, 3.62, 2.25 and 1.60 ms.
+  static constexpr uint32_t kLineCycles = 600;
+  static uint32_t pace(int stages, bool fp4, int ew) {
+    return static_cast<uint32_t>(stages) * (fp4 ? 640u : 560u) * 4u / 5u /
+           static_cast<uint32_t>(64 / ew + 1);
+  }
+
+  // PERSNP factors of a tile, loaded while the epilogue waits for the
+  // accumulator: inside the tile a load would wait behind the stores.  wi[t]:
+  // SNP i of the lane's store t; wj[k]: SNP j 32 k + lane of the warp's columns.
+  template <int NC>
+  struct Early {
+    float2 wi[4], wj[NC / 2];
+  };
+  template <int NC>
+  __device__ __forceinline__ static Early<NC> early(const Tally2Args &args, Tile2 sc, int quarter,
+                                                    int lane, int c0) {
+    Early<NC> e;
+    const bool on = args.ccc != nullptr && args.norm == CCC_NORM_PERSNP;
+    const float2 *w = reinterpret_cast<const float2 *>(args.w);
+    const int64_t i = static_cast<int64_t>(sc.I) * SNP_I + quarter * 16 + (lane >> 3);
+    const int64_t j = static_cast<int64_t>(sc.J) * SNP_J + c0 * 16 + lane;
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+      e.wi[t] = on && i + 4 * t < args.n_v ? __ldg(w + i + 4 * t) : make_float2(1.f, 1.f);
+#pragma unroll
+    for (int k = 0; k < NC / 2; ++k)
+      e.wj[k] = on && j + 32 * k < args.n_v ? __ldg(w + j + 32 * k) : make_float2(1.f, 1.f);
+    return e;
+  }
 
   // PRELOAD: all NC chunks are loaded, and the accumulator released, before
   // the first is processed.
   template <int NC, bool PRELOAD = false>
-  __device__ static void body(const Tally2Args &args, Tile2 sc, int quarter, int lane,
-                              uint32_t t_base, uint32_t release_cluster_bar, int c0,
-                              float *stage) {
-    if constexpr (PRELOAD) {
-      uint32_t pre[NC][32];
+  __device__ __forceinline__ static void body(const Tally2Args &args, Tile2 sc, int quarter,
+                                              int lane, uint32_t t_base,
+                                              uint32_t release_cluster_bar, int c0, float *stage,
+                                              const Early<NC> &e, bool more) {
+    if (args.ccc == nullptr)
+      run<NC, PRELOAD, TALLY>(args, sc, quarter, lane, t_base, release_cluster_bar, c0, stage, e, more);
+    else if (args.norm == CCC_NORM_PERSNP)
+      run<NC, PRELOAD, PERSNP>(args, sc, quarter, lane, t_base, release_cluster_bar, c0, stage, e, more);
+    else
+      run<NC, PRELOAD, JOINT>(args, sc, quarter, lane, t_base, release_cluster_bar, c0, stage, e, more);
+  }
+
+  // The lane's four SNPs i of a tile.
+  struct Rows {
+    char *out[4];       // tally address of table 0 of the row's first line, plus 16 l
+    int32_t rd[4];      // byte offset of that table in the ring
+    int32_t first[4];   // its j (relative to the warp's first) minus the row's first stored j
+    uint32_t width[4];  // j stored of this row
+    int64_t to_ccc;     // bytes from a tally to its values
+    int64_t p[4];       // checked builds: pair index of out[t]
+  };
+
+  __device__ __forceinline__ static Rows rows(const Tally2Args &args, int64_t ib, int64_t jb,
+                                              int jw, int lane) {
+    Rows r;
+    const int l = lane & 7, g = lane >> 3;
+    const int64_t n_v = args.n_v;
+    int64_t i = ib + g;
+    int64_t p = i * (2 * n_v - i - 1) / 2 - i - 1 + jb - args.pair0;  // pair (i, jb)
+    r.to_ccc = reinterpret_cast<char *>(args.ccc) - reinterpret_cast<char *>(args.tally);
+    const int hi = n_v - jb < jw ? static_cast<int>(n_v - jb) : jw;  // j past n_v are not stored
 #pragma unroll
-      for (int cc = 0; cc < NC; ++cc) tmem_ld_32x32b_x32(t_base + (c0 + cc) * 32, pre[cc]);
-      tmem_ld_wait();
+    for (int t = 0; t < 4; ++t) {
+      char *a = reinterpret_cast<char *>(args.tally) + 16 * p;
+      const int e = l - static_cast<int>((reinterpret_cast<uintptr_t>(a) >> 4) & 7);
+      const int unit = ((e & 15) ^ (4 * (t & 1) + g));  // low three bits permuted by the row's
+      r.out[t] = a + 16 * e;
+      r.rd[t] = (4 * t + g) * 256 + unit * 16;
+      const bool ok = i < n_v && i >= args.i_begin && i < args.i_end;
+      const int lo = i + 1 > jb ? static_cast<int>(i + 1 - jb) : 0;  // i < j
+      r.first[t] = e - lo;
+      r.width[t] = ok && hi > lo ? static_cast<uint32_t>(hi - lo) : 0u;
+      r.p[t] = p + e;
+      p += 4 * n_v - 4 * i - 14;  // pair (i + 4, jb)
+      i += 4;
+    }
+    return r;
+  }
+
+  // Piece q (8 SNPs j, 16 columns) of the lane's accumulator row into the ring.
+  template <Mode MODE>
+  __device__ __forceinline__ static void put(const uint32_t *v, int q, int lane, float2 wj,
+                                             char *ring, char *wring) {
+    const int il = lane >> 1;
+    char *const base = ring + il * 256 + (lane & 1) * 8 + (q & 1) * 128;
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      *reinterpret_cast<uint2 *>(base + ((k ^ (il & 7)) << 4)) = make_uint2(v[2 * k], v[2 * k + 1]);
+    if (MODE == PERSNP && (lane >> 3) == (q & 3))
+      *reinterpret_cast<float2 *>(wring + (q & 1) * 64 + (lane & 7) * 8) = wj;
+  }
+
+  // Line w of every row: tables 8 w - offset .. + 7, from pieces w - 1 and w.
+  template <Mode MODE>
+  __device__ __forceinline__ static void line(const Tally2Args &args, const Rows &r, int w,
+                                              const float2 (&wi)[4], const char *ring,
+                                              const char *wring, int g) {
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const int rd = r.rd[t] ^ (w & 1 ? 128 : 0);
+      const float4 x = *reinterpret_cast<const float4 *>(ring + rd);
+      const float2 r0 = make_float2(x.x, x.y), r1 = make_float2(x.z, x.w);
+      const bool ok = static_cast<uint32_t>(r.first[t] + 8 * w) < r.width[t] &&
+                      CCC_IN_BOUNDS(r.p[t] + 8 * w, args.out_len, args.status);
+      const int2 c0 = counts2(r0), c1 = counts2(r1);
+      // Streaming stores: the output passes through L2 once and should not
+      // evict the operand blocks that other tiles still read.
+      if (ok)
+        __stcs(reinterpret_cast<int4 *>(r.out[t] + 128 * w), make_int4(c0.x, c0.y, c1.x, c1.y));
+      if (MODE != TALLY) {
+        float2 wj = make_float2(1.f, 1.f);
+        if (MODE == PERSNP)
+          wj = *reinterpret_cast<const float2 *>(
+              wring + (((rd >> 1) & 0x78) ^ ((4 * (t & 1) + g) << 3)));
+        const float4 cv = ccc2_table<MODE == JOINT>(r0, r1, wi[t], wj, args.gamma);
+        if (ok) __stcs(reinterpret_cast<float4 *>(r.out[t] + r.to_ccc + 128 * w), cv);
+      }
+    }
+  }
+
+  template <int NC, bool PRELOAD, Mode MODE>
+  __device__ __forceinline__ static void run(const Tally2Args &args, Tile2 sc, int quarter,
+                                             int lane, uint32_t t_base,
+                                             uint32_t release_cluster_bar, int c0, float *stage,
+                                             const Early<NC> &e, bool more) {
+    constexpr int EW = 32 / NC;
+    const int ew = c0 / NC * 4 + quarter;
+    char *const ring = reinterpret_cast<char *>(stage);
+    char *const wring = ring + (EW - ew) * STAGE_BYTES_PER_WARP + ew * RING_BYTES_PER_WARP;
+    const int64_t ib = static_cast<int64_t>(sc.I) * SNP_I + quarter * 16;
+    const int64_t jb = static_cast<int64_t>(sc.J) * SNP_J + c0 * 16;
+    const int g = lane >> 3;
+    uint32_t v[PRELOAD ? NC : 1][32];
+    auto load = [&](int cc) { tmem_ld_32x32b_x32(t_base + (c0 + cc) * 32, v[PRELOAD ? cc : 0]); };
+    auto release = [&]() {
       tc_fence_before();
       mbar_arrive_cluster(release_cluster_bar);
+    };
+    auto piece = [&](int q) {
+      put<MODE>(v[PRELOAD ? q >> 1 : 0] + 16 * (q & 1), q, lane, e.wj[q >> 2], ring, wring);
+    };
+    load(0);
+    if (PRELOAD) {
 #pragma unroll
-      for (int cc = 0; cc < NC; ++cc) chunk(args, sc, quarter, lane, c0 + cc, pre[cc], stage);
-    } else {
-      for (int c = c0; c < c0 + NC; ++c) {
-        uint32_t v[32];
-        tmem_ld_32x32b_x32(t_base + c * 32, v);
-        tmem_ld_wait();
-        if (c == c0 + NC - 1) {
-          tc_fence_before();
-          mbar_arrive_cluster(release_cluster_bar);
-        }
-        chunk(args, sc, quarter, lane, c, v, stage);
-      }
+      for (int cc = 1; cc < NC; ++cc) load(cc);
     }
-  }
-
-  __device__ __forceinline__ static void chunk(const Tally2Args &args, Tile2 sc, int quarter,
-                                               int lane, int c, const uint32_t (&v)[32],
-                                               float *stage) {
-    at(args, static_cast<int64_t>(sc.I) * SNP_I + quarter * 16,
-       static_cast<int64_t>(sc.J) * SNP_J + c * 16, lane, v, stage);
-  }
-
-  // The 32 x 32 chunk of SNPs i ib .. ib + 15 (lanes) and j jb .. jb + 15 (columns).
-  __device__ __forceinline__ static void at(const Tally2Args &args, int64_t ib, int64_t jb,
-                                            int lane, const uint32_t (&v)[32], float *stage) {
-    const int64_t n_v = args.n_v;
-    const bool filter = args.hits != nullptr;
-    const bool want_ccc = filter || args.ccc != nullptr;
-    const bool persnp = args.norm == CCC_NORM_PERSNP;
-    const int jl = lane & 15;
-    const int64_t i0 = ib + (lane >> 4);
-    __syncwarp();  // the previous chunk's reads are done
-#pragma unroll
-    for (int k = 0; k < 32; ++k) stage[lane * STRIDE + k] = __uint_as_float(v[k]);
+    tmem_ld_wait();
+    if (PRELOAD || NC == 1) release();
+    __syncwarp();  // the previous tile's last lines have been read
+    piece(0);
+    piece(1);
     __syncwarp();
-    const int64_t j = jb + jl;
-    float wj0 = 1.f, wj1 = 1.f;
-    if (want_ccc && persnp && j < n_v) {
-      const float2 wj = __ldg(reinterpret_cast<const float2 *>(args.w) + j);
-      wj0 = wj.x;
-      wj1 = wj.y;
-    }
-#pragma unroll 2
-    for (int t = 0; t < 8; ++t) {
-      const int il = 2 * t + (lane >> 4);  // SNP i of this store within the chunk's 16
-      const int64_t i = i0 + 2 * t;
-      const float *r0 = stage + (2 * il) * STRIDE + 2 * jl;  // row (i, 0)
-      const float *r1 = r0 + STRIDE;                          // row (i, 1)
-      const int32_t r00 = __float2int_rn(r0[0]);
-      const int32_t r01 = __float2int_rn(r0[1]);
-      const int32_t r10 = __float2int_rn(r1[0]);
-      const int32_t r11 = __float2int_rn(r1[1]);
-      if (!(i < j && j < n_v && i >= args.i_begin && i < args.i_end)) continue;
-      const int64_t pidx = i * (2 * n_v - i - 1) / 2 - i - 1 + j - args.pair0;
-      if (!filter && !CCC_IN_BOUNDS(pidx, args.out_len, args.status)) continue;
-      if (!filter) __stcs(reinterpret_cast<int4 *>(args.tally) + pidx, make_int4(r00, r01, r10, r11));
-      if (!want_ccc) continue;
-      float wi0 = 1.f, wi1 = 1.f;
-      if (persnp) {
-        const float2 wi = __ldg(reinterpret_cast<const float2 *>(args.w) + i);
-        wi0 = wi.x;
-        wi1 = wi.y;
+    const Rows r = rows(args, ib, jb, NC * 16, lane);
+    // Line q starts no earlier than q pace cycles after the first, and the
+    // warps' first lines one after another (in an order of the cluster's own),
+    // where the next tile's MMAs leave time for it.
+    const uint32_t pace = more ? args.pace : 0u;
+    const uint32_t turn = (static_cast<uint32_t>(ew) + (blockIdx.x >> 1)) % EW;
+    const uint32_t begin = static_cast<uint32_t>(clock()) +
+                           (pace > kLineCycles ? (pace - kLineCycles) / EW * turn : 0u);
+    auto hold = [&](int q) {
+      while (static_cast<int32_t>(static_cast<uint32_t>(clock()) - begin - pace * q) < 0) {
       }
-      const bool skip = filter && persnp &&
-                        !may_exceed(r00, r01, r10, r11, wi0, wi1, wj0, wj1, args.threshold);
-      if (skip) continue;
-      const float4 cv = ccc2_values(r00, r01, r10, r11, wi0, wi1, wj0, wj1, args.norm, args.gamma);
-      if (filter)
-        filter_pair(args.hits, args.n_hits, args.cap, args.threshold, i, j, r00, r01, r10, r11, cv);
-      else
-        __stcs(reinterpret_cast<float4 *>(args.ccc) + pidx, cv);
+    };
+    hold(0);
+    line<MODE>(args, r, 0, e.wi, ring, wring, g);
+    hold(1);
+    line<MODE>(args, r, 1, e.wi, ring, wring, g);
+#pragma unroll
+    for (int cc = 1; cc < NC; ++cc) {
+      if (!PRELOAD) {
+        load(cc);
+        tmem_ld_wait();
+        if (cc == NC - 1) release();
+      }
+#pragma unroll
+      for (int q = 2 * cc; q < 2 * cc + 2; ++q) {
+        __syncwarp();  // line q - 1 has been read: piece q - 2 is free
+        hold(q);
+        piece(q);
+        __syncwarp();
+        line<MODE>(args, r, q, e.wi, ring, wring, g);
+      }
     }
+    line<MODE>(args, r, 2 * NC, e.wi, ring, wring, g);  // the rows' last, partial lines
   }
 };
 
-constexpr size_t pair_smem(int ew) { return tcp::smem_bytes(ew, Epi2Staged::STAGE_BYTES_PER_WARP); }
+constexpr size_t pair_smem(int ew) {
+  return tcp::smem_bytes(ew, Epi2Staged::STAGE_BYTES_PER_WARP) + Epi2Staged::extra_bytes(ew);
+}
 static_assert(pair_smem(8) <= 232448, "dynamic shared memory limit");
+
+// Threads of a 256-column SM-pair kernel.
+constexpr int pair_threads(int ew, bool fp4) { return fp4 ? tcp::SPLIT_THREADS : 64 + 32 * ew; }
+
+// Dynamic shared memory of a register-split kernel, and a check that it was
+// built with the registers that its warpgroups pass on: with fewer, the wait for
+// more would not end.
+template <class K>
+bool split_kernel_ready(K kernel, size_t smem) {
+  cudaFuncAttributes at;
+  return cudaFuncGetAttributes(&at, kernel) == cudaSuccess && at.numRegs == 168 &&
+         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              static_cast<int>(smem)) == cudaSuccess;
+}
 
 template <int EW>
 __global__ void __launch_bounds__(64 + 32 * EW, 1)
@@ -279,16 +421,21 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1)
 struct Epi2Pair {
   using Params = Tally2Args;
   static constexpr int STAGE_BYTES_PER_WARP = Epi2Staged::STAGE_BYTES_PER_WARP;
+  template <int NC>
+  __device__ __forceinline__ static auto early(const Params &args, const TriSchedPair &sc, int rank,
+                                               int quarter, int lane, int c0) {
+    return Epi2Staged::early<NC>(args, Tile2{2 * sc.I + rank, sc.J}, quarter, lane, c0);
+  }
   template <int NC, bool PRELOAD = false>
   __device__ static void tile(const Params &args, const TriSchedPair &sc, int rank, int quarter,
                               int lane, uint32_t t_base, uint32_t release_cluster_bar, int c0,
-                              float *stage) {
+                              float *stage, const Epi2Staged::Early<NC> &e, bool more) {
     if (args.hits != nullptr)  // thresholded output stores little: no staging
       Epi2::body<NC, true, PRELOAD>(args, Tile2{2 * sc.I + rank, sc.J}, quarter, lane, t_base,
                                     release_cluster_bar, c0);
     else
       Epi2Staged::body<NC, PRELOAD>(args, Tile2{2 * sc.I + rank, sc.J}, quarter, lane, t_base,
-                                    release_cluster_bar, c0, stage);
+                                    release_cluster_bar, c0, stage, e, more);
   }
 };
 
@@ -300,17 +447,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * EW, 1)
 }
 
 // FP4 (e2m1) operands: one accumulator, 8 epilogue warps that load their whole
-// quarter-half before releasing it (tcp::persistent_gemm_pair, FP4).  Each
-// epilogue thread holds 128 accumulator values.  The 10 warps of a CTA put 3
-// warps on two of the SM's four sub-partitions, whose register files hold 16K
-// registers each, so a thread may use at most 168 (3 x 32 x 168 <= 16,384):
-// that is what __launch_bounds__(320, 1) gives, with a few dozen bytes spilled.
-// A higher cap (183 registers, no spills) left no CTA resident.
+// quarter-half before releasing it (tcp::persistent_gemm_pair, FP4), each
+// thread holding 128 accumulator values; three warpgroups with a register split
+// (tcp::SPLIT_THREADS).
 // Default tile order of the FP4 kernels: groups of 16 column blocks (GB300,
 // 20,000 x 16,384: 3.76 ms against 3.80 with 8, 3.82 with 32; 200,000 x 4,096
 // thresholded: 121 against 127 ms with 8, 125 with 32).
 constexpr int kFp4Group = 16;
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * tcp::FP4_EW, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tcp::SPLIT_THREADS, 1)
     k_tally2_tc_pair_fp4(const __grid_constant__ CUtensorMap tm, const Tally2Args args,
                          TriSched::Params sp, int nkb) {
   tcp::persistent_gemm_pair<TriSchedPair, Epi2Pair, tcp::FP4_EW, false, true>(&tm, sp, args, nkb,
@@ -360,10 +504,14 @@ struct Epi2Rect {
   static_assert(TAIL == 16 && CHUNKS == 7, "chunks 0-3, 4-6 and a 16-column tail");
   static_assert(STAGE_BYTES_PER_WARP % 16 == 0, "16-byte staged rows");
 
+  template <int NC>
+  __device__ __forceinline__ static tcp::NoEarly early(const Params &, const Sched &, int, int, int, int) {
+    return {};
+  }
   template <int NC, bool PRELOAD>
   __device__ static void tile(const Params &args, const Sched &sc, int rank, int quarter, int lane,
                               uint32_t t_base, uint32_t release_cluster_bar, int c0,
-                              float *stage) {
+                              float *stage, tcp::NoEarly, bool) {
     static_assert(!PRELOAD, "two accumulators: each warp releases after its last load");
     const int half = c0 / NC;
     const int64_t ib = static_cast<int64_t>(2 * sc.I + rank) * SNP_I;  // the CTA's first SNP i
@@ -526,10 +674,14 @@ static_assert(rect_smem() <= 232448, "dynamic shared memory limit");
 struct Epi2Split {
   using Params = Tally2Args;
   static constexpr int STAGE_BYTES_PER_WARP = 0;
+  template <int NC>
+  __device__ __forceinline__ static tcp::NoEarly early(const Params &, const SplitSchedPair &, int, int, int, int) {
+    return {};
+  }
   template <int NC, bool PRELOAD = false>
   __device__ static void tile(const Params &args, const SplitSchedPair &sc, int rank, int quarter,
                               int lane, uint32_t t_base, uint32_t release_cluster_bar, int c0,
-                              float *) {
+                              float *, tcp::NoEarly, bool) {
     body<NC, PRELOAD>(args, Tile2{2 * sc.I + rank, sc.J}, quarter, lane, t_base,
                       release_cluster_bar, c0);
   }
@@ -587,7 +739,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * EW, 1)
   tcp::persistent_gemm_pair<SplitSchedPair, Epi2Split, EW, true>(&tm, sp, args, nkb, args.status);
 }
 
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * tcp::FP4_EW, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tcp::SPLIT_THREADS, 1)
     k_tally2_tc_pair_split_fp4(const __grid_constant__ CUtensorMap tm, const Tally2Args args,
                                SplitSchedPair::Params sp, int nkb) {
   tcp::persistent_gemm_pair<SplitSchedPair, Epi2Split, tcp::FP4_EW, true, true>(&tm, sp, args, nkb,
@@ -615,7 +767,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * EW + 32 * 
 }
 
 constexpr size_t packed_smem(int ew) {
-  return tcp::pk::smem_bytes(ew, Epi2Staged::STAGE_BYTES_PER_WARP);
+  return tcp::pk::smem_bytes(ew, Epi2Staged::STAGE_BYTES_PER_WARP) + Epi2Staged::extra_bytes(ew);
 }
 static_assert(packed_smem(8) <= 232448, "dynamic shared memory limit");
 
@@ -702,17 +854,23 @@ struct BatchSchedPair : BatchSchedT<TriSchedPair> {};
 struct EpiBatchPair {
   using Params = BatchParams;
   static constexpr int STAGE_BYTES_PER_WARP = Epi2Staged::STAGE_BYTES_PER_WARP;
+  template <int NC>
+  __device__ __forceinline__ static auto early(const Params &bp, const BatchSchedPair &sc, int rank,
+                                               int quarter, int lane, int c0) {
+    return Epi2Staged::early<NC>(bp.p[sc.p].args, Tile2{2 * sc.t.I + rank, sc.t.J}, quarter, lane,
+                                 c0);
+  }
   template <int NC, bool PRELOAD = false>
   __device__ static void tile(const Params &bp, const BatchSchedPair &sc, int rank, int quarter,
                               int lane, uint32_t t_base, uint32_t release_cluster_bar, int c0,
-                              float *stage) {
+                              float *stage, const Epi2Staged::Early<NC> &e, bool more) {
     const BatchPanel &q = bp.p[sc.p];
     if (q.split > 1)  // a K part: partial tallies added into the zeroed output
       Epi2Split::body<NC, PRELOAD>(q.args, Tile2{2 * sc.t.I + rank, sc.t.J}, quarter, lane, t_base,
                                    release_cluster_bar, c0);
     else
       Epi2Staged::body<NC, PRELOAD>(q.args, Tile2{2 * sc.t.I + rank, sc.t.J}, quarter, lane,
-                                    t_base, release_cluster_bar, c0, stage);
+                                    t_base, release_cluster_bar, c0, stage, e, more);
   }
 };
 
@@ -724,7 +882,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * EW, 1)
                                                              bp.p[0].args.status);
 }
 
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * tcp::FP4_EW, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tcp::SPLIT_THREADS, 1)
     k_tally2_tc_pair_batched_fp4(const __grid_constant__ BatchMaps maps,
                                  const __grid_constant__ BatchParams bp) {
   tcp::persistent_gemm_pair<BatchSchedPair, EpiBatchPair, tcp::FP4_EW, false, true>(
@@ -823,9 +981,7 @@ int launch_tally2_tc_pair_batched(const Tally2Args *args, const uint8_t *const *
         cudaFuncSetAttribute(k_tally2_tc_pair_batched<8>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(pair_smem(8))) != cudaSuccess ||
-        cudaFuncSetAttribute(k_tally2_tc_pair_batched_fp4,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(pair_smem(tcp::FP4_EW))) != cudaSuccess)
+        !split_kernel_ready(k_tally2_tc_pair_batched_fp4, pair_smem(tcp::FP4_EW)))
       return CCC_ECUDA;
     attr_set[dev] = true;
   }
@@ -856,6 +1012,7 @@ int launch_tally2_tc_pair_batched(const Tally2Args *args, const uint8_t *const *
   }
   if (units == 0) return CCC_OK;
   const int ew = fp4 ? tcp::FP4_EW : epilogue_warps(static_cast<int>(kw / static_cast<double>(units)));
+  for (int k = 0; k < n; ++k) bp.p[k].args.pace = Epi2Staged::pace(bp.p[k].nkb, fp4, ew);
   static int max_clusters[kMaxDevices][3] = {};
   int &mc = max_clusters[dev][fp4 ? 2 : ew == 4 ? 0 : 1];
   if (mc == 0) {
@@ -866,7 +1023,7 @@ int launch_tally2_tc_pair_batched(const Tally2Args *args, const uint8_t *const *
     attr.val.clusterDim.y = 1;
     attr.val.clusterDim.z = 1;
     cfg.gridDim = dim3(static_cast<unsigned>(num_sms), 1, 1);
-    cfg.blockDim = dim3(static_cast<unsigned>(64 + 32 * ew), 1, 1);
+    cfg.blockDim = dim3(static_cast<unsigned>(pair_threads(ew, fp4)), 1, 1);
     cfg.dynamicSmemBytes = pair_smem(ew);
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
@@ -881,8 +1038,7 @@ int launch_tally2_tc_pair_batched(const Tally2Args *args, const uint8_t *const *
   const int64_t clusters = units < mc ? units : mc;
   const int grid = static_cast<int>(2 * clusters);
   if (fp4)
-    k_tally2_tc_pair_batched_fp4<<<grid, 64 + 32 * tcp::FP4_EW, pair_smem(tcp::FP4_EW), s>>>(maps,
-                                                                                           bp);
+    k_tally2_tc_pair_batched_fp4<<<grid, tcp::SPLIT_THREADS, pair_smem(tcp::FP4_EW), s>>>(maps, bp);
   else if (ew == 4)
     k_tally2_tc_pair_batched<4><<<grid, 64 + 32 * 4, pair_smem(4), s>>>(maps, bp);
   else
@@ -940,8 +1096,9 @@ int launch_tally2_tc_batched(const Tally2Args *args, const uint8_t *const *ops,
   return note_launch();
 }
 
-int launch_tally2_tc_pair(const Tally2Args &a, const uint8_t *op, int64_t rows_pad, int64_t kpad,
+int launch_tally2_tc_pair(const Tally2Args &args, const uint8_t *op, int64_t rows_pad, int64_t kpad,
                           int num_sms, cudaStream_t s, bool fp4) {
+  Tally2Args a = args;
   static bool attr_set[kMaxDevices] = {};
   const int dev = current_device();
   if (dev < 0) return CCC_ECUDA;
@@ -950,8 +1107,7 @@ int launch_tally2_tc_pair(const Tally2Args &a, const uint8_t *op, int64_t rows_p
                              static_cast<int>(pair_smem(4))) != cudaSuccess ||
         cudaFuncSetAttribute(k_tally2_tc_pair<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(pair_smem(8))) != cudaSuccess ||
-        cudaFuncSetAttribute(k_tally2_tc_pair_fp4, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(pair_smem(tcp::FP4_EW))) != cudaSuccess ||
+        !split_kernel_ready(k_tally2_tc_pair_fp4, pair_smem(tcp::FP4_EW)) ||
         cudaFuncSetAttribute(k_tally2_tc_pair_fp4w, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(rect_smem())) != cudaSuccess)
       return CCC_ECUDA;
@@ -1013,6 +1169,7 @@ int launch_tally2_tc_pair(const Tally2Args &a, const uint8_t *op, int64_t rows_p
   const int64_t tiles = tc2_pair_tiles(a.n_v, sp.I0, sp.I1);
   if (tiles == 0) return CCC_OK;
   const int ew = fp4 ? tcp::FP4_EW : epilogue_warps(nkb);
+  a.pace = Epi2Staged::pace(nkb, fp4, ew);
   // Persistent grid: as many SM pairs as can be resident at once.
   int &mc = max_clusters[dev][fp4 ? 2 : ew == 4 ? 0 : 1];
   if (mc == 0) {
@@ -1023,7 +1180,7 @@ int launch_tally2_tc_pair(const Tally2Args &a, const uint8_t *op, int64_t rows_p
     attr.val.clusterDim.y = 1;
     attr.val.clusterDim.z = 1;
     cfg.gridDim = dim3(static_cast<unsigned>(num_sms), 1, 1);
-    cfg.blockDim = dim3(static_cast<unsigned>(64 + 32 * ew), 1, 1);
+    cfg.blockDim = dim3(static_cast<unsigned>(pair_threads(ew, fp4)), 1, 1);
     cfg.dynamicSmemBytes = pair_smem(ew);
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
@@ -1038,7 +1195,7 @@ int launch_tally2_tc_pair(const Tally2Args &a, const uint8_t *op, int64_t rows_p
   const int64_t clusters = tiles < mc ? tiles : mc;
   const int grid = static_cast<int>(2 * clusters);
   if (fp4)
-    k_tally2_tc_pair_fp4<<<grid, 64 + 32 * tcp::FP4_EW, pair_smem(tcp::FP4_EW), s>>>(tm, a, sp, nkb);
+    k_tally2_tc_pair_fp4<<<grid, tcp::SPLIT_THREADS, pair_smem(tcp::FP4_EW), s>>>(tm, a, sp, nkb);
   else if (ew == 4)
     k_tally2_tc_pair<4><<<grid, 64 + 32 * 4, pair_smem(4), s>>>(tm, a, sp, nkb);
   else
@@ -1052,14 +1209,12 @@ int launch_tally2_tc_pair_split(const Tally2Args &a, const uint8_t *op, int64_t 
   const int dev = current_device();
   if (dev < 0) return CCC_ECUDA;
   int &max_clusters = max_clusters_dev[dev][fp4 ? 1 : 0];
-  const int threads = 64 + 32 * (fp4 ? tcp::FP4_EW : 4);
+  const int threads = pair_threads(4, fp4);
   const size_t smem = tcp::SMEM_BYTES;
   if (max_clusters == 0) {
     if (cudaFuncSetAttribute(k_tally2_tc_pair_split<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(smem)) != cudaSuccess ||
-        cudaFuncSetAttribute(k_tally2_tc_pair_split_fp4,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(smem)) != cudaSuccess)
+        !split_kernel_ready(k_tally2_tc_pair_split_fp4, smem))
       return CCC_ECUDA;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr;

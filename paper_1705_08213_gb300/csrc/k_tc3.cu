@@ -151,29 +151,19 @@ struct Epi3 {
           __stcs(reinterpret_cast<int2 *>(args.tally) + 4 * t + ab, make_int2(r0, r1));
           if (want_ccc) {
             const int32_t n8 = q0 + q1;
-            float2 out = make_float2(0.f, 0.f);
-            if (n8 != 0) {
-              const float d = static_cast<float>(n8);
-              float fi = wi, fj = wj, fk0, fk1;
-              if (persnp) {
-                const float2 wk = __ldg(reinterpret_cast<const float2 *>(args.w) + k);
-                fk0 = wk.x;
-                fk1 = wk.y;
-              } else {
-                fi = joint_factor(ra, d, args.gamma);
-                fj = joint_factor(rb, d, args.gamma);
-                fk0 = joint_factor(q0, d, args.gamma);
-                fk1 = joint_factor(q1, d, args.gamma);
-              }
-              if (persnp) {
-                const float inv = __frcp_rn(d);
-                const float wij = __fmul_rn(fi, fj);
-                out.x = ccc3_persnp(r0, inv, wij, fk0);
-                out.y = ccc3_persnp(r1, inv, wij, fk1);
-              } else {
-                out.x = __fmul_rn(__fmul_rn(__fmul_rn(__fdiv_rn(static_cast<float>(r0), d), fi), fj), fk0);
-                out.y = __fmul_rn(__fmul_rn(__fmul_rn(__fdiv_rn(static_cast<float>(r1), d), fi), fj), fk1);
-              }
+            const float d = n8 == 0 ? 1.f : static_cast<float>(n8);
+            const float inv = rcp_count(d);
+            const float2 r = make_float2(static_cast<float>(r0), static_cast<float>(r1));
+            float2 out;
+            if (persnp) {
+              const float2 wk = __ldg(reinterpret_cast<const float2 *>(args.w) + k);
+              out = mul2(mul2(mul2(r, both(inv)), both(__fmul_rn(wi, wj))), wk);
+            } else {
+              const float fi = joint_factor(static_cast<float>(ra), d, inv, args.gamma);
+              const float fj = joint_factor(static_cast<float>(rb), d, inv, args.gamma);
+              const float2 fk = joint_factors(
+                  make_float2(static_cast<float>(q0), static_cast<float>(q1)), d, inv, args.gamma);
+              out = mul2(mul2(mul2(div_count(r, d, inv), both(fi)), both(fj)), fk);
             }
             __stcs(reinterpret_cast<float2 *>(args.ccc) + 4 * t + ab, out);
           }

@@ -538,30 +538,20 @@ __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
             const int32_t q0 = c0 + __shfl_xor_sync(0xffffffffu, c0, 1);
             const int32_t q1 = c1 + __shfl_xor_sync(0xffffffffu, c1, 1);
             if (ok) {
-              float4 out = make_float4(0.f, 0.f, 0.f, 0.f);
-              if (n8 != 0) {
-                const float dn = static_cast<float>(n8);
-                float fi = wi, fj0 = wj0, fj1 = wj1, fk0 = wk[kk].x, fk1 = wk[kk].y;
-                if (!persnp) {
-                  fi = joint_factor(own, dn, gamma);
-                  fj0 = joint_factor(rb0, dn, gamma);
-                  fj1 = joint_factor(rb1, dn, gamma);
-                  fk0 = joint_factor(q0, dn, gamma);
-                  fk1 = joint_factor(q1, dn, gamma);
-                }
-                if (persnp) {
-                  const float inv = __frcp_rn(dn);
-                  const float g0 = __fmul_rn(fi, fj0), g1 = __fmul_rn(fi, fj1);
-                  out.x = ccc3_persnp(tv.x, inv, g0, fk0);
-                  out.y = ccc3_persnp(tv.y, inv, g0, fk1);
-                  out.z = ccc3_persnp(tv.z, inv, g1, fk0);
-                  out.w = ccc3_persnp(tv.w, inv, g1, fk1);
-                } else {
-                  out.x = __fmul_rn(__fmul_rn(__fmul_rn(__fdiv_rn(static_cast<float>(tv.x), dn), fi), fj0), fk0);
-                  out.y = __fmul_rn(__fmul_rn(__fmul_rn(__fdiv_rn(static_cast<float>(tv.y), dn), fi), fj0), fk1);
-                  out.z = __fmul_rn(__fmul_rn(__fmul_rn(__fdiv_rn(static_cast<float>(tv.z), dn), fi), fj1), fk0);
-                  out.w = __fmul_rn(__fmul_rn(__fmul_rn(__fdiv_rn(static_cast<float>(tv.w), dn), fi), fj1), fk1);
-                }
+              const float dn = n8 == 0 ? 1.f : static_cast<float>(n8);
+              const float inv = rcp_count(dn);
+              const float2 f0 = make_float2(static_cast<float>(tv.x), static_cast<float>(tv.y));
+              const float2 f1 = make_float2(static_cast<float>(tv.z), static_cast<float>(tv.w));
+              float4 out;
+              if (persnp) {
+                out = ccc3_persnp(f0, f1, inv, mul2(both(wi), make_float2(wj0, wj1)), wk[kk]);
+              } else {
+                const float fi = joint_factor(static_cast<float>(own), dn, inv, gamma);
+                const float2 fj = joint_factors(
+                    make_float2(static_cast<float>(rb0), static_cast<float>(rb1)), dn, inv, gamma);
+                const float2 fk = joint_factors(
+                    make_float2(static_cast<float>(q0), static_cast<float>(q1)), dn, inv, gamma);
+                out = ccc3_joint(f0, f1, dn, inv, fi, fj, fk);
               }
               __stcs(ccc_out + 2 * t + a, out);
             }
@@ -1103,30 +1093,20 @@ __global__ void __launch_bounds__(wide::kThreads, 1) __cluster_dims__(2, 1, 1)
                 q1 = c1 + __shfl_xor_sync(0xffffffffu, c1, 1);
               }
               if (ok) {
-                float4 out = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (n8 != 0) {
-                  const float dn = static_cast<float>(n8);
-                  float fi = wi, fj0 = wj0, fj1 = wj1, fk0 = wk[kk].x, fk1 = wk[kk].y;
-                  if (!persnp) {
-                    fi = joint_factor(own, dn, gamma);
-                    fj0 = joint_factor(rb0, dn, gamma);
-                    fj1 = joint_factor(rb1, dn, gamma);
-                    fk0 = joint_factor(q0, dn, gamma);
-                    fk1 = joint_factor(q1, dn, gamma);
-                  }
-                  if (persnp) {
-                    const float inv = __frcp_rn(dn);
-                    const float g0 = __fmul_rn(fi, fj0), g1 = __fmul_rn(fi, fj1);
-                    out.x = ccc3_persnp(tv.x, inv, g0, fk0);
-                    out.y = ccc3_persnp(tv.y, inv, g0, fk1);
-                    out.z = ccc3_persnp(tv.z, inv, g1, fk0);
-                    out.w = ccc3_persnp(tv.w, inv, g1, fk1);
-                  } else {
-                    out.x = __fmul_rn(__fmul_rn(__fmul_rn(__fdiv_rn(static_cast<float>(tv.x), dn), fi), fj0), fk0);
-                    out.y = __fmul_rn(__fmul_rn(__fmul_rn(__fdiv_rn(static_cast<float>(tv.y), dn), fi), fj0), fk1);
-                    out.z = __fmul_rn(__fmul_rn(__fmul_rn(__fdiv_rn(static_cast<float>(tv.z), dn), fi), fj1), fk0);
-                    out.w = __fmul_rn(__fmul_rn(__fmul_rn(__fdiv_rn(static_cast<float>(tv.w), dn), fi), fj1), fk1);
-                  }
+                const float dn = n8 == 0 ? 1.f : static_cast<float>(n8);
+                const float inv = rcp_count(dn);
+                const float2 f0 = make_float2(static_cast<float>(tv.x), static_cast<float>(tv.y));
+                const float2 f1 = make_float2(static_cast<float>(tv.z), static_cast<float>(tv.w));
+                float4 out;
+                if (persnp) {
+                  out = ccc3_persnp(f0, f1, inv, mul2(both(wi), make_float2(wj0, wj1)), wk[kk]);
+                } else {
+                  const float fi = joint_factor(static_cast<float>(own), dn, inv, gamma);
+                  const float2 fj = joint_factors(
+                      make_float2(static_cast<float>(rb0), static_cast<float>(rb1)), dn, inv, gamma);
+                  const float2 fk = joint_factors(
+                      make_float2(static_cast<float>(q0), static_cast<float>(q1)), dn, inv, gamma);
+                  out = ccc3_joint(f0, f1, dn, inv, fi, fj, fk);
                 }
                 __stcs(ccc_out + 2 * t + a, out);
               }

@@ -50,11 +50,29 @@ constexpr uint32_t IDESC_FP4 = idesc_e2m1_f32(256, 256, true);
 constexpr uint32_t SF_COL = 256;
 constexpr uint32_t SF_ONE_UE8M0 = 0x7F7F7F7Fu;
 constexpr int FP4_EW = 8;
+// Register split of the one-accumulator pipeline: an epilogue thread holds 128
+// accumulator values, and the 168 registers that 10 warps leave each thread (3
+// warps on a sub-partition of 16K registers) make it spill and serialise.  So
+// three warpgroups are launched at 168 registers a thread (12 warps, 64,512 of the
+// 65,536): the one of the TMA and MMA threads (two of its warps idle) gives
+// up all but 56, and the two of the epilogue take 224: 56 + 2 x 224 = 3 x 168.
+constexpr int SPLIT_THREADS = 384;
+constexpr int SPLIT_REGS_MAIN = 56;
+constexpr int SPLIT_REGS_EPI = 224;
+static_assert(SPLIT_REGS_MAIN + 2 * SPLIT_REGS_EPI == 3 * 168, "the launch's registers");
+template <int REGS>
+__device__ __forceinline__ void regs_down() {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS));
+}
+template <int REGS>
+__device__ __forceinline__ void regs_up() {
+  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS));
+}
 constexpr size_t SMEM_BYTES = 1024 + static_cast<size_t>(STAGES) * STAGE_BYTES + NUM_BARS * 8 + 64;
 // Dynamic shared memory of a kernel whose epilogue warps each stage
 // `stage_bytes` (Epi::STAGE_BYTES_PER_WARP) after the barriers.
 constexpr size_t smem_bytes(int epi_warps, int stage_bytes) {
-  return SMEM_BYTES + (stage_bytes > 0 ? 16 + static_cast<size_t>(epi_warps) * stage_bytes : 0);
+  return SMEM_BYTES + (stage_bytes > 0 ? 256 + static_cast<size_t>(epi_warps) * stage_bytes : 0);
 }
 // The same for tiles of NB < 256 columns (B rows NB / 2 per CTA).
 constexpr size_t smem_bytes_nb(int nb, int epi_warps, int stage_bytes) {
@@ -166,16 +184,23 @@ __device__ __forceinline__ void mma_commit_pair(uint32_t bar, uint16_t mask) {
       : "memory");
 }
 
+// For epilogues that load nothing early.
+struct NoEarly {};
+
 // Sched: as for tc::persistent_gemm, in units of 256-row tiles; a_row/b_row
 // give the first row of the tile (the CTA adds 128 r); map_index() selects the
 // tile's tensor map in tm[]; the tile's K stages are k_begin() ..
 // k_begin() + k_blocks(nkb) - 1.
-// Epi: template <int NC> static void tile(const Params&, const Sched&, int rank,
+// Epi: template <int NC> static T early(const Params&, const Sched&, int rank,
+//        int quarter, int lane, int c0): what the tile's epilogue needs from
+//        global memory, loaded before the accumulator is waited for;
+//      template <int NC> static void tile(const Params&, const Sched&, int rank,
 //        int quarter, int lane, uint32_t t_base, uint32_t release_cluster_bar,
-//        int c0, float *stage); the release arrives at a cluster address;
+//        int c0, float *stage, const T&, bool more); the release arrives at a
+//        cluster address; more: the cluster has another tile after this one;
 //        static constexpr int STAGE_BYTES_PER_WARP: shared memory each epilogue
 //        warp may use at `stage` (the kernel is launched with
-//        smem_bytes(EW, STAGE_BYTES_PER_WARP)).
+//        smem_bytes(EW, STAGE_BYTES_PER_WARP)), slice 4 (c0 / NC) + quarter.
 // KBLK: the operand is stored K-block-major, [nkb][rows][128 bytes], behind a
 // 3-D tensor map (x = byte, y = row, z = K block), so that each 128-row box is
 // one contiguous 16 KB run.
@@ -200,6 +225,9 @@ __device__ __forceinline__ void persistent_gemm_pair(const CUtensorMap *tm,
   constexpr int B_BYTES_T = NBH * BK;     // B bytes per CTA and K stage
   constexpr int STAGE_BYTES_T = A_BYTES + B_BYTES_T;
   constexpr int NACC = FP4 && NB == 256 ? 1 : 2;  // accumulator buffers
+  constexpr bool SPLIT_REGS = NACC == 1;          // launched with SPLIT_THREADS threads
+  constexpr int E0 = SPLIT_REGS ? 4 : 2;          // first epilogue warp
+  static_assert(!SPLIT_REGS || 32 * (E0 + EW) == SPLIT_THREADS, "three warpgroups");
   constexpr uint32_t SF_T = NACC == 1 ? SF_COL : 2u * NB;  // FP4 scale-factor columns
   static_assert(NB == 256 || (FP4 && !KBLK && NB % 16 == 0 && NB >= 128 &&
                               SF_T + 32 <= static_cast<uint32_t>(TMEM_COLS)),
@@ -211,8 +239,11 @@ __device__ __forceinline__ void persistent_gemm_pair(const CUtensorMap *tm,
   uint64_t *bars = reinterpret_cast<uint64_t *>(sB + STAGES * B_BYTES_T);
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + NUM_BARS);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
-  float *const stage_base = reinterpret_cast<float *>(
-      (reinterpret_cast<uintptr_t>(tmem_slot) + 64 + 15) & ~static_cast<uintptr_t>(15));
+  // An offset from the shared array, not an integer made a pointer: the compiler
+  // then sees a shared address (LDS, STS) instead of a generic one, which would
+  // go through the global load path, behind the epilogue's stores.
+  float *const stage_base =
+      reinterpret_cast<float *>(smem_raw + (((smem_u32(tmem_slot) + 64u + 255u) & ~255u) - raw));
 
   constexpr int EPI_THREADS = tc::Epilogue<EW>::THREADS;
   static_assert(!FP4 || EW == FP4_EW, "the FP4 epilogue holds 4 chunks per thread");
@@ -256,7 +287,7 @@ __device__ __forceinline__ void persistent_gemm_pair(const CUtensorMap *tm,
     // Scale factors 1.0 in both CTAs' columns SF_T .. SF_T + 31 (every
     // byte), written by the first four epilogue warps, one lane quarter each,
     // before the leader's first MMA reads them.
-    if (warp >= 2 && warp < 6) {
+    if (warp >= E0 && warp < E0 + 4) {
       uint32_t v[32];
 #pragma unroll
       for (int k = 0; k < 32; ++k) v[k] = SF_ONE_UE8M0;
@@ -269,8 +300,9 @@ __device__ __forceinline__ void persistent_gemm_pair(const CUtensorMap *tm,
     tc_fence_after();
   }
 
-  if (warp == 0) {
-    if (lane == 0) {
+  if (warp < E0) {
+    if constexpr (SPLIT_REGS) regs_down<SPLIT_REGS_MAIN>();
+    if (warp == 0 && lane == 0) {
       // ---------------- TMA producer (both CTAs)
       int stage = 0;
       uint32_t phase = 0;
@@ -321,8 +353,7 @@ __device__ __forceinline__ void persistent_gemm_pair(const CUtensorMap *tm,
         }
       }
     }
-  } else if (warp == 1) {
-    if (lane == 0 && leader) {
+    if (warp == 1 && lane == 0 && leader) {
       // ---------------- MMA issuer (leader CTA)
       int stage = 0;
       uint32_t phase = 0;
@@ -367,22 +398,29 @@ __device__ __forceinline__ void persistent_gemm_pair(const CUtensorMap *tm,
       mbar_wait_timeout(drain_bar, 0);
     }
   } else {
+    if constexpr (SPLIT_REGS) regs_up<SPLIT_REGS_EPI>();
     // ---------------- epilogue (both CTAs)
     const int quarter = warp & 3;
+    const int half = (warp - E0) >> 2;
     constexpr int NC = tc::Epilogue<EW>::CHUNKS_PER_WARP;
-    const int c0 = ((warp - 2) >> 2) * NC;
+    const int c0 = half * NC;
     int lt = 0;
-    Sched sc;
-    for (sc.init(sp, cstart); sc.valid; sc.advance(cstep), ++lt) {
+    Sched sc, next;
+    for (sc.init(sp, cstart); sc.valid; sc = next, ++lt) {
+      next = sc;
+      next.advance(cstep);
       const int acc = NACC == 1 ? 0 : (lt & 1);
       const uint32_t acc_phase = NACC == 1 ? (lt & 1) : ((lt >> 1) & 1);
+      const auto early = Epi::template early<NC>(ep, sc, static_cast<int>(rank), quarter, lane, c0);
       const bool ok = mbar_wait_bounded(tfull_bar(acc), acc_phase, status, abort_flag);
       if (!__all_sync(0xffffffffu, ok)) break;
       tc_fence_after();
       const uint32_t t_base = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + acc * NB;
       Epi::template tile<NC, NACC == 1>(ep, sc, static_cast<int>(rank), quarter, lane, t_base,
                                         map_to_rank(tempty_bar(acc), 0), c0,
-                                        stage_base + (warp - 2) * (Epi::STAGE_BYTES_PER_WARP / 4));
+                                        stage_base + (4 * half + quarter) *
+                                                         (Epi::STAGE_BYTES_PER_WARP / 4),
+                                        early, next.valid);
     }
   }
 
@@ -428,7 +466,7 @@ constexpr int NUM_BARS = 2 * P_STAGES + 3 * OP_STAGES + 5;
 constexpr size_t SMEM_BYTES = 1024 + static_cast<size_t>(OP_STAGES) * STAGE_BYTES +
                               static_cast<size_t>(P_STAGES) * P_BYTES + NUM_BARS * 8 + 64;
 constexpr size_t smem_bytes(int epi_warps, int stage_bytes) {
-  return SMEM_BYTES + (stage_bytes > 0 ? 16 + static_cast<size_t>(epi_warps) * stage_bytes : 0);
+  return SMEM_BYTES + (stage_bytes > 0 ? 256 + static_cast<size_t>(epi_warps) * stage_bytes : 0);
 }
 static_assert(A_BYTES == B_BYTES, "one operand stage size");
 static_assert((2 * SNPS * (BK / 16)) % (WPT * 32) == 0, "converter tasks per stage");
@@ -496,8 +534,11 @@ __device__ __forceinline__ void persistent_gemm_pair_packed(const CUtensorMap *t
   uint64_t *bars = reinterpret_cast<uint64_t *>(sP + P_STAGES * P_BYTES);
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + pk::NUM_BARS);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
-  float *const stage_base = reinterpret_cast<float *>(
-      (reinterpret_cast<uintptr_t>(tmem_slot) + 64 + 15) & ~static_cast<uintptr_t>(15));
+  // An offset from the shared array, not an integer made a pointer: the compiler
+  // then sees a shared address (LDS, STS) instead of a generic one, which would
+  // go through the global load path, behind the epilogue's stores.
+  float *const stage_base =
+      reinterpret_cast<float *>(smem_raw + (((smem_u32(tmem_slot) + 64u + 255u) & ~255u) - raw));
 
   constexpr int EPI_THREADS = tc::Epilogue<EW>::THREADS;
   const int warp = threadIdx.x >> 5;
@@ -637,12 +678,14 @@ __device__ __forceinline__ void persistent_gemm_pair_packed(const CUtensorMap *t
     // ---------------- epilogue (both CTAs)
     const int quarter = warp & 3;
     constexpr int NC = tc::Epilogue<EW>::CHUNKS_PER_WARP;
-    const int c0 = ((warp - 2) >> 2) * NC;
+    const int half = (warp - 2) >> 2;
+    const int c0 = half * NC;
     int lt = 0;
     Sched sc;
     for (sc.init(sp, cstart); sc.valid; sc.advance(cstep), ++lt) {
       const int acc = lt & 1;
       const uint32_t acc_phase = (lt >> 1) & 1;
+      const auto early = Epi::template early<NC>(ep, sc, static_cast<int>(rank), quarter, lane, c0);
       const bool ok = mbar_wait_bounded(tfull_bar(acc), acc_phase, status, abort_flag);
       if (!__all_sync(0xffffffffu, ok)) break;
       tc_fence_after();
@@ -650,7 +693,8 @@ __device__ __forceinline__ void persistent_gemm_pair_packed(const CUtensorMap *t
           tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + acc * ACC_COLS;
       Epi::template tile<NC>(ep, sc, static_cast<int>(rank), quarter, lane, t_base,
                              map_to_rank(tempty_bar(acc), 0), c0,
-                             stage_base + (warp - 2) * (Epi::STAGE_BYTES_PER_WARP / 4));
+                             stage_base + (4 * half + quarter) * (Epi::STAGE_BYTES_PER_WARP / 4),
+                             early, false);
     }
   } else {
     // ---------------- converters (both CTAs)
