@@ -629,6 +629,7 @@ static int prep_3way(Run3 &R, bool want_ccc, int64_t j_last) {
   a2.i_end = je - 1;
   a2.pair0 = 0;
   a2.out_len = pairs_in_rows(p->n_v, 0, p->n_v);  // the table holds every pair
+  a2.pack16 = tc3_class_table16(p->n_f);
   return launch_tally2_tc_pair(a2, op, R.L.rows_pad, R.L.kpad, R.dev.sms, s, R.fp4);
 }
 
@@ -648,8 +649,8 @@ static int slabs_3way(Run3 &R) {
     // Per batch of slabs: the compacted rows of the individuals with v_j
     // missing, the masked rows, the class kernel.  Batches alternate between
     // L.halves buffers; with two, batch b + 1 is prepared on a side stream
-    // (which first waits for everything already queued on s) while batch b's
-    // tally kernel runs.
+    // (which first waits for everything already queued on s), in the tail of
+    // batch b's tally kernel.
     if (jb >= je) return CCC_OK;
     uint8_t *op = at<uint8_t>(o, L.op);
     int32_t *rtab = at<int32_t>(o, L.rtab);

@@ -106,6 +106,9 @@ struct Tally2Args {
   float threshold = 0.f;
   // Column blocks per L2 group of the tensor-core tile order (0 = default 8).
   int32_t group = 0;
+  // SM-pair kernels: tallies below 2^16 stored as four 16-bit numbers per pair
+  // (8 bytes, tally an array of them; no CCC values).
+  bool pack16 = false;
   // Cycles between the output lines of a tile in the SM-pair kernels (set by
   // their launches; 0 = stored as fast as they come).
   uint32_t pace = 0;
@@ -209,7 +212,9 @@ int launch_tally3_fused(const Tally3Args &a, const uint64_t *geno, int64_t ld, c
 //                    n_v) rows of kpad bytes) into op from row mrow0 on, op's
 //                    first rows being the count matrix R;
 //   launch_tally3_class  the tallies, with the 2-way tallies rtab ([pair][4],
-//                    pairs i < k with i < j1 - 1).
+//                    pairs i < k with i < j1 - 1; as 16-bit numbers when
+//                    tc3_class_table16(n_f)).
+bool tc3_class_table16(int64_t n_f);
 int64_t tc3_class_cap();
 int64_t tc3_class_cbuf_rows(int64_t n_slabs, int64_t n_v);
 int64_t tc3_class_mask_rows(int64_t j0, int64_t j1, int64_t n_v);

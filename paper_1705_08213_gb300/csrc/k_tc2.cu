@@ -190,7 +190,9 @@ struct Epi2Staged {
   static constexpr int RING_BYTES_PER_WARP = 16 * 8;     // the factors w_j of the ring's 16 j
   static constexpr size_t extra_bytes(int ew) { return static_cast<size_t>(ew) * RING_BYTES_PER_WARP; }
 
-  enum Mode { TALLY, PERSNP, JOINT };
+  // PACK16: the tallies alone, as four 16-bit numbers of 8 bytes a pair (the
+  // table r_ik of the 3-way classes; args.pack16), a line being 64 bytes.
+  enum Mode { TALLY, PACK16, PERSNP, JOINT };
 
   // Cycles from line to line that spread a tile's lines (2 NC + 1, NC = 32 / ew
   // chunks per warp) over about 4/5 of the MMAs of the next tile, K stages of
@@ -236,7 +238,10 @@ struct Epi2Staged {
                                               int lane, uint32_t t_base,
                                               uint32_t release_cluster_bar, int c0, float *stage,
                                               const Early<NC> &e, bool more) {
-    if (args.ccc == nullptr)
+    if (args.pack16)
+      run<NC, PRELOAD, PACK16>(args, sc, quarter, lane, t_base, release_cluster_bar, c0, stage, e,
+                               more);
+    else if (args.ccc == nullptr)
       run<NC, PRELOAD, TALLY>(args, sc, quarter, lane, t_base, release_cluster_bar, c0, stage, e, more);
     else if (args.norm == CCC_NORM_PERSNP)
       run<NC, PRELOAD, PERSNP>(args, sc, quarter, lane, t_base, release_cluster_bar, c0, stage, e, more);
@@ -254,6 +259,7 @@ struct Epi2Staged {
     int64_t p[4];       // checked builds: pair index of out[t]
   };
 
+  template <int REC>  // bytes of a pair
   __device__ __forceinline__ static Rows rows(const Tally2Args &args, int64_t ib, int64_t jb,
                                               int jw, int lane) {
     Rows r;
@@ -265,10 +271,10 @@ struct Epi2Staged {
     const int hi = n_v - jb < jw ? static_cast<int>(n_v - jb) : jw;  // j past n_v are not stored
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
-      char *a = reinterpret_cast<char *>(args.tally) + 16 * p;
-      const int e = l - static_cast<int>((reinterpret_cast<uintptr_t>(a) >> 4) & 7);
+      char *a = reinterpret_cast<char *>(args.tally) + REC * p;
+      const int e = l - static_cast<int>((reinterpret_cast<uintptr_t>(a) / REC) & 7);
       const int unit = ((e & 15) ^ (4 * (t & 1) + g));  // low three bits permuted by the row's
-      r.out[t] = a + 16 * e;
+      r.out[t] = a + REC * e;
       r.rd[t] = (4 * t + g) * 256 + unit * 16;
       const bool ok = i < n_v && i >= args.i_begin && i < args.i_end;
       const int lo = i + 1 > jb ? static_cast<int>(i + 1 - jb) : 0;  // i < j
@@ -309,6 +315,13 @@ struct Epi2Staged {
       const int2 c0 = counts2(r0), c1 = counts2(r1);
       // Streaming stores: the output passes through L2 once and should not
       // evict the operand blocks that other tiles still read.
+      if (MODE == PACK16) {
+        if (ok)
+          *reinterpret_cast<uint2 *>(r.out[t] + 64 * w) =
+              make_uint2(static_cast<uint32_t>(c0.x | (c0.y << 16)),
+                         static_cast<uint32_t>(c1.x | (c1.y << 16)));
+        continue;
+      }
       if (ok)
         __stcs(reinterpret_cast<int4 *>(r.out[t] + 128 * w), make_int4(c0.x, c0.y, c1.x, c1.y));
       if (MODE != TALLY) {
@@ -354,7 +367,7 @@ struct Epi2Staged {
     piece(0);
     piece(1);
     __syncwarp();
-    const Rows r = rows(args, ib, jb, NC * 16, lane);
+    const Rows r = rows<MODE == PACK16 ? 8 : 16>(args, ib, jb, NC * 16, lane);
     // Line q starts no earlier than q pace cycles after the first, and the
     // warps' first lines one after another (in an order of the cluster's own),
     // where the next tile's MMAs leave time for it.
@@ -397,17 +410,6 @@ static_assert(pair_smem(8) <= 232448, "dynamic shared memory limit");
 
 // Threads of a 256-column SM-pair kernel.
 constexpr int pair_threads(int ew, bool fp4) { return fp4 ? tcp::SPLIT_THREADS : 64 + 32 * ew; }
-
-// Dynamic shared memory of a register-split kernel, and a check that it was
-// built with the registers that its warpgroups pass on: with fewer, the wait for
-// more would not end.
-template <class K>
-bool split_kernel_ready(K kernel, size_t smem) {
-  cudaFuncAttributes at;
-  return cudaFuncGetAttributes(&at, kernel) == cudaSuccess && at.numRegs == 168 &&
-         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              static_cast<int>(smem)) == cudaSuccess;
-}
 
 template <int EW>
 __global__ void __launch_bounds__(64 + 32 * EW, 1)
@@ -981,7 +983,7 @@ int launch_tally2_tc_pair_batched(const Tally2Args *args, const uint8_t *const *
         cudaFuncSetAttribute(k_tally2_tc_pair_batched<8>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(pair_smem(8))) != cudaSuccess ||
-        !split_kernel_ready(k_tally2_tc_pair_batched_fp4, pair_smem(tcp::FP4_EW)))
+        !tcp::split_kernel_ready(k_tally2_tc_pair_batched_fp4, pair_smem(tcp::FP4_EW)))
       return CCC_ECUDA;
     attr_set[dev] = true;
   }
@@ -1107,7 +1109,7 @@ int launch_tally2_tc_pair(const Tally2Args &args, const uint8_t *op, int64_t row
                              static_cast<int>(pair_smem(4))) != cudaSuccess ||
         cudaFuncSetAttribute(k_tally2_tc_pair<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(pair_smem(8))) != cudaSuccess ||
-        !split_kernel_ready(k_tally2_tc_pair_fp4, pair_smem(tcp::FP4_EW)) ||
+        !tcp::split_kernel_ready(k_tally2_tc_pair_fp4, pair_smem(tcp::FP4_EW)) ||
         cudaFuncSetAttribute(k_tally2_tc_pair_fp4w, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(rect_smem())) != cudaSuccess)
       return CCC_ECUDA;
@@ -1214,7 +1216,7 @@ int launch_tally2_tc_pair_split(const Tally2Args &a, const uint8_t *op, int64_t 
   if (max_clusters == 0) {
     if (cudaFuncSetAttribute(k_tally2_tc_pair_split<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(smem)) != cudaSuccess ||
-        !split_kernel_ready(k_tally2_tc_pair_split_fp4, smem))
+        !tcp::split_kernel_ready(k_tally2_tc_pair_split_fp4, smem))
       return CCC_ECUDA;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr;

@@ -157,7 +157,7 @@ struct Epi3 {
             float2 out;
             if (persnp) {
               const float2 wk = __ldg(reinterpret_cast<const float2 *>(args.w) + k);
-              out = mul2(mul2(mul2(r, both(inv)), both(__fmul_rn(wi, wj))), wk);
+              out = mul2(r, mul2(mul2(both(inv), wk), both(__fmul_rn(wi, wj))));
             } else {
               const float fi = joint_factor(static_cast<float>(ra), d, inv, args.gamma);
               const float fj = joint_factor(static_cast<float>(rb), d, inv, args.gamma);

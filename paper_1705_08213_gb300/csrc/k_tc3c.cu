@@ -102,7 +102,7 @@ __device__ __forceinline__ bool mbar_wait_cluster_bounded(uint32_t bar, uint32_t
 }
 
 // D-slot accesses with an L2 evict-last policy: each slot is written and read
-// back by the same thread one tile later, while the tiles' outputs stream
+// back by the same warp one tile later, while the tiles' outputs stream
 // through L2 (evict-first stores); without the hint the slots were evicted and
 // written back to DRAM between the two.
 __device__ __forceinline__ uint64_t l2_evict_last_policy() {
@@ -115,10 +115,19 @@ __device__ __forceinline__ void st_l2_keep(uint32_t *p, uint32_t v, uint64_t pol
   asm volatile("st.global.L2::cache_hint.b32 [%0], %1, %2;" ::"l"(p), "r"(v), "l"(pol) : "memory");
 }
 
-__device__ __forceinline__ uint32_t ld_l2_keep(const uint32_t *p, uint64_t pol) {
-  uint32_t v;
-  asm volatile("ld.global.L2::cache_hint.b32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(pol) : "memory");
-  return v;
+__device__ __forceinline__ void ld2_keep_if(uint2 &v, bool ok, const uint32_t *p, uint64_t pol) {
+  asm volatile(
+      "{\n.reg .pred q;\nsetp.ne.s32 q, %4, 0;\n"
+      "@q ld.global.L2::cache_hint.v2.b32 {%0, %1}, [%2], %3;\n}"
+      : "+r"(v.x), "+r"(v.y)
+      : "l"(p), "l"(pol), "r"(static_cast<int>(ok)));
+}
+
+__device__ __forceinline__ void ld2_if(uint2 &v, bool ok, const uint2 *p) {
+  asm volatile(
+      "{\n.reg .pred q;\nsetp.ne.s32 q, %3, 0;\n@q ld.global.nc.v2.b32 {%0, %1}, [%2];\n}"
+      : "+r"(v.x), "+r"(v.y)
+      : "l"(p), "r"(static_cast<int>(ok)));
 }
 
 // P(x) = sum_{j < x} min(j, n_v - 1 - j): SNPs on the masked side of the
@@ -148,14 +157,24 @@ struct ClassSchedT {
   int mt, nt, m, n;
   bool valid;
 
-  __device__ void set_slab() {
-    mt = static_cast<int>(cdiv(j, kSnpI));
-    nt = static_cast<int>(cdiv(n_v - 1 - j, SNPK));
+  // 32-bit arithmetic throughout (n_v <= 65,535 and, per launch, fewer than
+  // 2^31 tiles): every warp walks the tiles by itself, and the slabs of a small
+  // panel hold only a few each.
+  __device__ __forceinline__ void set_slab() {
+    mt = (j + kSnpI - 1) / kSnpI;
+    nt = static_cast<int>(static_cast<unsigned>(n_v - 1 - j + SNPK - 1) / SNPK);
   }
-  __device__ void skip_empty() {
+  // The first slab from j on that holds more than `skip` tiles, less those of the slabs before it.
+  __device__ __forceinline__ void seek(int skip) {
     while (j < j1) {
       set_slab();
-      if (mt > 0 && nt > 0) return;
+      const int tiles = mt * nt;
+      if (skip < tiles) {
+        m = static_cast<int>(static_cast<unsigned>(skip) / static_cast<unsigned>(nt));
+        n = skip - m * nt;
+        return;
+      }
+      skip -= tiles;
       ++j;
     }
     valid = false;
@@ -169,23 +188,10 @@ struct ClassSchedT {
     missing_ = p.missing;
     m = n = 0;
     valid = true;
-    skip_empty();
-    advance(start);
+    seek(static_cast<int>(start));
   }
-  __device__ void advance(int64_t step) {
-    while (valid && step > 0) {
-      const int64_t pos = static_cast<int64_t>(m) * nt + n;
-      const int64_t rem = static_cast<int64_t>(mt) * nt - 1 - pos;
-      if (step <= rem) {
-        m = static_cast<int>((pos + step) / nt);
-        n = static_cast<int>((pos + step) % nt);
-        return;
-      }
-      step -= rem + 1;
-      ++j;
-      m = n = 0;
-      skip_empty();
-    }
+  __device__ __forceinline__ void advance(int64_t step) {
+    if (valid) seek(m * nt + n + static_cast<int>(step));
   }
   __device__ int i0() const { return kSnpI * m; }
   __device__ int k0() const { return j + 1 + SNPK * n; }
@@ -206,7 +212,7 @@ struct ClassSchedT {
   __device__ int d_blocks(bool *full) const {
     const int c = missing();
     *full = c > kCap;
-    return *full ? nkb : static_cast<int>(cdiv(c, KBI));
+    return *full ? nkb : (c + KBI - 1) / KBI;
   }
 };
 using ClassSched = ClassSchedT<kSnpK>;
@@ -240,7 +246,7 @@ __device__ __forceinline__ void class_masks(uint32_t w, bool missing_mode, uint3
 
 struct ClassArgs {
   Tally3Args t;
-  const int32_t *rtab;  // 2-way tallies [pair][4]
+  const int32_t *rtab;  // 2-way tallies [pair][4]; wide tiles: as 16-bit numbers
   uint32_t *dscratch;   // wide tiles: [cta][2][k][lane] D counts
 };
 
@@ -544,7 +550,7 @@ __global__ void __launch_bounds__(kThreads, 1) __cluster_dims__(2, 1, 1)
               const float2 f1 = make_float2(static_cast<float>(tv.z), static_cast<float>(tv.w));
               float4 out;
               if (persnp) {
-                out = ccc3_persnp(f0, f1, inv, mul2(both(wi), make_float2(wj0, wj1)), wk[kk]);
+                out = ccc3_persnp(f0, f1, mul2(both(inv), wk[kk]), mul2(both(wi), make_float2(wj0, wj1)));
               } else {
                 const float fi = joint_factor(static_cast<float>(own), dn, inv, gamma);
                 const float2 fj = joint_factors(
@@ -598,32 +604,215 @@ constexpr int kTile = 128 * kBK;                  // 128 rows x 128 bytes
 constexpr int kStageBytes = 2 * kTile;            // A + B per CTA
 constexpr int kDWords = 128 * 128;                // per tile: [k (0..127)][lane] x (u16 c = 0, u16 c = 1)
 constexpr int kMaxCtas = 256;                     // CTAs the D scratch is sized for
-// Epilogue: 2 warps per TMEM lane quarter; warp g of a quarter takes the
-// 8-SNP chunks c = g, g + 2, ... of the tile's 16 (12 warps measured slower:
-// their register cap of 146 cost more than the added overlap gave).
+// Epilogue: 2 warps per TMEM lane quarter (16 SNPs i); warp h of a quarter takes
+// the SNPs k from 64 h on (64, or what the tile has), 8-SNP chunks in order.
+// (12 warps measured slower: their register cap cost more than the added
+// overlap gave.)  The T accumulators go through a ring of two chunks per warp
+// in shared memory, so that the stores are whole 128-byte lines (4 triples) of
+// the slab's rows: see Epi3.
 constexpr int kEpiWarps = 8;
-// The 2-way tallies r_ik of an epilogue warp's next chunk (its 16 SNPs i x 8
-// SNPs k, 128 bytes per i) are copied into shared memory with asynchronous
-// 16-byte copies (cp.async, each warp instruction 4 whole rows) while it works
-// on the current chunk: rows 144 bytes apart, so that the lanes' 8-byte reads
-// of one k are free of bank conflicts.  GB300, 1,536 x 8,192: class kernels
-// 14.24 -> 13.7 ms against one 8-byte load per lane and k from the 2-way table
-// (16 rows per warp load); a second buffer (prefetching two chunks ahead)
-// measured the same.  Five operand stages measured as fast as six here and
-// leave shared memory for the preparation kernels of the next batch.
-constexpr int kRowStride = 144;
-constexpr int kRbufBytes = 16 * kRowStride;
+constexpr int kHalfK = 64;
+constexpr int kRingBytes = 16 * 256;  // 16 SNPs i x 16 k x 2 alleles x (c = 0, 1)
+constexpr int kWringBytes = 16 * 8;   // the factors w_k of the ring's 16 k
 constexpr int kNumBars = 2 * kStages + 2 + 2 + 3;  // full, empty, tfull, tempty, dready, ddone, drain
 constexpr size_t kSmem = 1024 + static_cast<size_t>(kStages) * kStageBytes + kNumBars * 8 + 64 +
-                         16 + static_cast<size_t>(kEpiWarps) * kRbufBytes;
-constexpr int kGroups = kEpiWarps / 4;
-constexpr int kThreads = 64 + 32 * kEpiWarps;
+                         256 + static_cast<size_t>(kEpiWarps) * (kRingBytes + kWringBytes);
+constexpr int kThreads = tcp::SPLIT_THREADS;
+constexpr int kE0 = 4;  // first epilogue warp
+constexpr int kRegsMain = 88, kRegsEpi = 208;
+static_assert(kRegsMain + 2 * kRegsEpi == 3 * 168, "the launch's registers");
 static_assert(kSmem <= 232448, "dynamic shared memory limit");
 static_assert(2 * Cfg<true>::kN + 32 <= 512 && kSfCol == 2 * Cfg<true>::kN, "FP4 TMEM layout");
 static_assert(Cfg<true>::kN % 16 == 0 && Cfg<true>::kN / 2 <= 128, "FP4 tile: N per CTA in the B box");
 }  // namespace wide
 
 constexpr int64_t kWideMaxNf = 16383;  // 4 n_f < 2^16
+
+// 32 bytes of a triple's eight numbers if ok (predicated, no branch), in one
+// store (VEC: the address is a multiple of 32) or two.
+template <bool VEC>
+__device__ __forceinline__ void store8(bool ok, char *p, int4 x, int4 y) {
+  if (VEC)
+    asm volatile(
+        "{\n.reg .pred q;\nsetp.ne.s32 q, %9, 0;\n"
+        "@q st.global.cs.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n}" ::"l"(p),
+        "r"(x.x), "r"(x.y), "r"(x.z), "r"(x.w), "r"(y.x), "r"(y.y), "r"(y.z), "r"(y.w),
+        "r"(static_cast<int>(ok)));
+  else
+    asm volatile(
+        "{\n.reg .pred q;\nsetp.ne.s32 q, %9, 0;\n"
+        "@q st.global.cs.v4.b32 [%0], {%1, %2, %3, %4};\n"
+        "@q st.global.cs.v4.b32 [%0 + 16], {%5, %6, %7, %8};\n}" ::"l"(p),
+        "r"(x.x), "r"(x.y), "r"(x.z), "r"(x.w), "r"(y.x), "r"(y.y), "r"(y.z), "r"(y.w),
+        "r"(static_cast<int>(ok)));
+}
+
+__device__ __forceinline__ int4 bits4(float4 v) {
+  return make_int4(__float_as_int(v.x), __float_as_int(v.y), __float_as_int(v.z), __float_as_int(v.w));
+}
+
+// Epilogue of the wide tiles.  Accumulator lane (i, a), columns (k, c): the warp
+// writes eight k at a time into its ring, as 16 bytes per (i, k), and reads them
+// back so that lane 8 g + l of store t holds triple l of two 128-byte lines of
+// the output row of SNP i = 4 t + g, all of its eight numbers: a warp store covers
+// eight whole lines.  The rows of a slab start at any triple, so two lines may
+// lie across two chunks by the row's own offset.  What bounds it is the number
+// of instructions (two epilogue warps per scheduler) and the stores; stored as
+// they came from the accumulator, by allele, a warp store was 16 pieces of 32
+// bytes and a triple took two lanes of about 95 instructions, now one of about
+// 75: the counts stay in the floats of the accumulator, the table's and D's
+// 16-bit numbers are subtracted two at a time, and no value crosses lanes.
+// GB300, class kernels per call: 1,536 x 8,192 13.6 -> 11.4 ms (8.3 without its
+// stores, 7.9 without its loads either, 6.5 of MMAs); calls: 301 x 2,001 JOINT
+// 279 -> 213 us, 1,000 x 1,000 JOINT -> 2.95 ms (3.6 TB/s).
+template <int MODE>
+struct Epi3 {
+  char *out[4];          // tally address of the lane's triple in the row's first lines
+  const uint2 *r[4];     // its packed r_ik
+  int32_t doff[4];       // its words (a = 0, 1) in the D slot
+  int32_t e[4];          // its k (relative to the warp's first)
+  uint32_t width[4];     // k stored of this row (0: none)
+  int32_t rd[4];         // byte offset in the ring of its T
+  int64_t to_ccc;
+  bool vec;                // both arrays are aligned to 32 bytes
+  int64_t tix[4], pix[4];  // checked builds: triple and pair index of e[t]
+  float2 wij[4][2];        // PERSNP: w_i(a) w_j(0), w_i(a) w_j(1) (products())
+  float2 wj;
+
+  struct Fetch {
+    uint2 r[4], d[4];
+  };
+
+  // Rows of the warp: SNPs ib .. ib + 15 and k from kf on, kn of them in the tile.
+  __device__ __forceinline__ void init(const ClassArgs &args, int64_t j, int64_t ib, int64_t kf,
+                                       int kn, int quarter, int half, int lane, int64_t s_begin) {
+    const int64_t n_v = args.t.n_v;
+    const int g = lane >> 3, l = lane & 7;
+    const int64_t span = n_v - 1 - j;
+    int64_t i = ib + g;
+    int64_t t0 = slab_offset_dev(j, n_v) - s_begin + i * span - (j + 1) + kf;  // triple (i, j, kf)
+    int64_t p0 = i * (2 * n_v - i - 1) / 2 - i - 1 + kf;                       // pair (i, kf)
+    to_ccc = reinterpret_cast<char *>(args.t.ccc) - reinterpret_cast<char *>(args.t.tally);
+    vec = ((reinterpret_cast<uintptr_t>(args.t.tally) | reinterpret_cast<uintptr_t>(args.t.ccc)) & 31) == 0;
+    const int hi = n_v - kf < kn ? static_cast<int>(n_v - kf) : kn;
+    const float2 *w2 = reinterpret_cast<const float2 *>(args.t.w);
+    wj = MODE == 1 ? __ldg(w2 + j) : make_float2(1.f, 1.f);
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      char *const row = reinterpret_cast<char *>(args.t.tally) + 32 * t0;
+      e[t] = l - static_cast<int>((reinterpret_cast<uintptr_t>(row) >> 5) & 3);
+      out[t] = row + 32 * e[t];
+      r[t] = reinterpret_cast<const uint2 *>(args.rtab) + p0 + e[t];
+      const int il = 4 * t + g;
+      doff[t] = (wide::kHalfK * half + e[t]) * 128 + quarter * 32 + 2 * il;
+      rd[t] = il * 256 + (((e[t] & 15) ^ (il & 7)) << 4);
+      const bool ok = i < j;
+      width[t] = ok && hi > 0 ? static_cast<uint32_t>(hi) : 0u;
+      tix[t] = t0 + e[t];
+      pix[t] = p0 + e[t];
+      if (MODE == 1) wij[t][0] = ok ? __ldg(w2 + i) : make_float2(1.f, 1.f);
+      t0 += 4 * span;
+      p0 += 4 * n_v - 4 * i - 14;  // pair (i + 4, kf)
+      i += 4;
+    }
+  }
+
+  // After init's loads have had time to arrive.
+  __device__ __forceinline__ void products() {
+#pragma unroll
+    for (int t = 0; t < 4 && MODE == 1; ++t) {
+      wij[t][1] = mul2(both(wij[t][0].y), wj);
+      wij[t][0] = mul2(both(wij[t][0].x), wj);
+    }
+  }
+
+  __device__ __forceinline__ bool in(int t, int k) const {
+    return static_cast<uint32_t>(e[t] + k) < width[t];
+  }
+
+  // The table's and D's words of the lines at k: predicated loads into registers
+  // whose other values are never stored, and no branch, so that the loads stay
+  // in flight across the chunk before theirs.  Without D, f.d stays as it was: 0.
+  __device__ __forceinline__ void fetch(Fetch &f, const ClassArgs &args, int k, bool has_d,
+                                        const uint32_t *slot, uint64_t pol) const {
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const bool ok = in(t, k) && CCC_IN_BOUNDS(pix[t] + k, args.t.n_v * (args.t.n_v - 1) / 2,
+                                                args.t.status);
+      ld2_if(f.r[t], ok, r[t] + k);
+      ld2_keep_if(f.d[t], ok && has_d, slot + doff[t] + 128 * k, pol);
+    }
+  }
+
+  // Columns of eight k of the lane's accumulator row into the ring's chunk at byte side (0, 128).
+  __device__ __forceinline__ static void put(const uint32_t (&x)[16], int side, int lane, char *ring) {
+    const int il = lane >> 1;
+    char *const row = ring + il * 256 + 8 * (lane & 1) + side;
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      *reinterpret_cast<uint2 *>(row + ((k ^ (il & 7)) << 4)) = make_uint2(x[2 * k], x[2 * k + 1]);
+  }
+
+  // r_ik - D of allele a, both c at once (no borrow: D counts a subset of r_ik).
+  __device__ __forceinline__ static float2 rest(uint32_t r, uint32_t d) {
+    const uint32_t u = r - d;
+    return add2(make_float2(__uint_as_float((u & 0xFFFFu) | 0x4B000000u),
+                            __uint_as_float((u >> 16) | 0x4B000000u)),
+                both(-8388608.f));
+  }
+
+  // The lines at k, every row's eight triples; side: of the ring's chunk that starts at k.
+  __device__ __forceinline__ void line(const ClassArgs &args, int k, int side, const Fetch &f,
+                                       const char *ring, const char *wring) const {
+    if (vec)
+      lines<true>(args, k, side, f, ring, wring);
+    else
+      lines<false>(args, k, side, f, ring, wring);
+  }
+  template <bool VEC>
+  __device__ __forceinline__ void lines(const ClassArgs &args, int k, int side, const Fetch &f,
+                                       const char *ring, const char *wring) const {
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const float4 T = *reinterpret_cast<const float4 *>(ring + (rd[t] ^ side));
+      const bool ok = in(t, k) && CCC_IN_BOUNDS(tix[t] + k, args.t.out_len, args.t.status);
+      const float2 t0 = make_float2(T.x, T.y), t1 = make_float2(T.z, T.w);
+      const float2 u0 = rest(f.r[t].x, f.d[t].x), u1 = rest(f.r[t].y, f.d[t].y);
+      // r^{a b c} over c: [a][b] = u_a + T_a, u_a - T_a
+      const float2 r00 = add2(u0, t0), r01 = fma2(t0, both(-1.f), u0);
+      const float2 r10 = add2(u1, t1), r11 = fma2(t1, both(-1.f), u1);
+      char *const dst = out[t] + 32 * k;
+      const int2 c00 = counts2(r00), c01 = counts2(r01), c10 = counts2(r10), c11 = counts2(r11);
+      store8<VEC>(ok, dst, make_int4(c00.x, c00.y, c01.x, c01.y),
+                  make_int4(c10.x, c10.y, c11.x, c11.y));
+      if constexpr (MODE != 0) {
+        const float2 half_c = add2(u0, u1);                  // half the sums over a, b
+        const float half_n = __fadd_rn(half_c.x, half_c.y);  // 4 n_ijk
+        const float d = fmaxf(__fadd_rn(half_n, half_n), 1.f);
+        const float inv = rcp_count(d);
+        float4 v0, v1;
+        if constexpr (MODE == 1) {
+          const float2 wk =
+              *reinterpret_cast<const float2 *>(wring + (((e[t] & 15) << 3) ^ (side >> 1)));
+          const float2 gk = mul2(both(inv), wk);
+          v0 = ccc3_persnp(r00, r01, gk, wij[t][0]);
+          v1 = ccc3_persnp(r10, r11, gk, wij[t][1]);
+        } else {
+          const float gamma = args.t.gamma;
+          const float2 b0 = add2(r00, r10), b1 = add2(r01, r11);
+          const float2 fi = joint_factors(
+              mul2(both(2.f), make_float2(__fadd_rn(u0.x, u0.y), __fadd_rn(u1.x, u1.y))), d, inv, gamma);
+          const float2 fj = joint_factors(
+              make_float2(__fadd_rn(b0.x, b0.y), __fadd_rn(b1.x, b1.y)), d, inv, gamma);
+          const float2 fk = joint_factors(add2(half_c, half_c), d, inv, gamma);
+          v0 = ccc3_joint(r00, r01, d, inv, fi.x, fj, fk);
+          v1 = ccc3_joint(r10, r11, d, inv, fi.y, fj, fk);
+        }
+        store8<VEC>(ok, dst + to_ccc, bits4(v0), bits4(v1));
+      }
+    }
+  }
+};
 
 // MODE 0: tallies only; 1: tallies and CCC, PERSNP; 2: tallies and CCC, JOINT.
 // FP4: e2m1 operands (see wide::Cfg).
@@ -700,7 +889,7 @@ __global__ void __launch_bounds__(wide::kThreads, 1) __cluster_dims__(2, 1, 1)
   if (FP4) {
     // Scale factors 1.0 (UE8M0) in columns kSfCol .. kSfCol + 31 of both CTAs,
     // one lane quarter per epilogue warp, before the leader's first MMA.
-    if (warp >= 2 && warp < 6) {
+    if (warp >= wide::kE0 && warp < wide::kE0 + 4) {
       uint32_t v[32];
 #pragma unroll
       for (int k = 0; k < 32; ++k) v[k] = tcp::SF_ONE_UE8M0;
@@ -719,8 +908,9 @@ __global__ void __launch_bounds__(wide::kThreads, 1) __cluster_dims__(2, 1, 1)
   // that the epilogue has finished the buffer it reuses (7/8 of a tile).
   const int ins = (7 * nkb) / 8;
 
-  if (warp == 0) {
-    if (lane == 0) {
+  if (warp < wide::kE0) {
+    tcp::regs_down<wide::kRegsMain>();
+    if (warp == 0 && lane == 0) {
       // ---------------- TMA producer (both CTAs)
       int stage = 0;
       uint32_t phase = 0;
@@ -799,8 +989,7 @@ __global__ void __launch_bounds__(wide::kThreads, 1) __cluster_dims__(2, 1, 1)
         }
       }
     }
-  } else if (warp == 1) {
-    if (lane == 0 && leader) {
+    if (warp == 1 && lane == 0 && leader) {
       // ---------------- MMA issuer (leader CTA)
       const uint64_t dA0 = smem_desc_sw128(smem_u32(sA));
       const uint64_t dB0 = smem_desc_sw128(smem_u32(sB));
@@ -899,7 +1088,7 @@ __global__ void __launch_bounds__(wide::kThreads, 1) __cluster_dims__(2, 1, 1)
       }
       tcp::mma_commit_pair(drain_bar, 0x1);
       mbar_wait_timeout(drain_bar, 0);
-    } else if (lane == 0) {
+    } else if (warp == 1 && lane == 0) {
       // ---------------- follower: forward the epilogue's releases to the leader
       int dcount = 0;
       Sched sc;
@@ -926,201 +1115,119 @@ __global__ void __launch_bounds__(wide::kThreads, 1) __cluster_dims__(2, 1, 1)
       }
     }
   } else {
+    tcp::regs_up<wide::kRegsEpi>();
     // ---------------- epilogue (both CTAs)
     const int quarter = warp & 3;
-    const int group = (warp - 2) >> 2;  // chunks group, group + kGroups, ...
+    const int half = (warp - wide::kE0) >> 2;  // k from wide::kHalfK * half on
     const int L = quarter * 32 + lane;  // TMEM lane = A row of this CTA
-    const int a = L & 1;
-    const int32_t *__restrict__ rtab = args.rtab;
-    const float *__restrict__ wv = args.t.w;
-    int4 *__restrict__ tally_out = reinterpret_cast<int4 *>(args.t.tally);
-    float4 *__restrict__ ccc_out = reinterpret_cast<float4 *>(args.t.ccc);
-    constexpr bool want_ccc = MODE != 0;
-    constexpr bool persnp = MODE == 1;
-    const float gamma = args.t.gamma;
     const int64_t s_begin = slab_offset_dev(args.t.j_begin, n_v);
     const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
     const uint64_t keep_pol = l2_evict_last_policy();
-    // r_ik staging of this warp: row il (SNP i = the warp's first + il) at
-    // rbuf + il kRowStride, pair (i, kc + kk) at + 16 kk.
-    const uint32_t rbuf =
-        static_cast<uint32_t>(((smem_u32(tmem_slot) + 64 + 15) & ~15u) +
-                              static_cast<uint32_t>(warp - 2) * wide::kRbufBytes);
-    // Asynchronous copies of the r_ik of chunk c of tile t for this warp's rows:
-    // lane copies pair lane % 8 of rows lane / 8 + 4 m, m = 0..3, 16 bytes each;
-    // none for rows i >= j or pairs past n_v.
-    auto issue_rows = [&](const Sched &t, int c) {
-      const int64_t kk = t.k0() + 8 * c + (lane & 7);  // this lane's pair column, in every piece
-      int64_t ii = t.i0() + 64 * static_cast<int64_t>(rank) + 16 * quarter + (lane >> 3);
-      int64_t pb = ii * (2 * n_v - ii - 1) / 2 - ii - 1;  // pair (ii, k) at pb + k
-      uint32_t dst = rbuf + static_cast<uint32_t>(lane >> 3) * wide::kRowStride +
-                     16u * static_cast<uint32_t>(lane & 7);
-#pragma unroll 1
-      for (int m = 0; m < 4; ++m) {  // rows lane / 8 + 4 m
-        if (ii < t.j && kk < n_v)
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst),
-                       "l"(rtab + 4 * (pb + kk))
-                       : "memory");
-        pb += 4 * n_v - 4 * ii - 14;  // pb(ii + 4) = pb(ii) + sum of n_v - i - 2 over 4 rows
-        ii += 4;
-        dst += 4 * wide::kRowStride;
-      }
-      asm volatile("cp.async.commit_group;" ::: "memory");
-    };
+    char *const rings =
+        reinterpret_cast<char *>(smem_raw) + (((smem_u32(tmem_slot) + 64u + 255u) & ~255u) - raw);
+    const int slice = 4 * half + quarter;
+    char *const ring = rings + slice * wide::kRingBytes;
+    char *const wring = rings + kEpiWarps * wide::kRingBytes + slice * wide::kWringBytes;
+    const int c_first = half * (wide::kHalfK / 8);  // the warp's 8-k chunks
+    const int chunks = half == 0 ? wide::kHalfK / 8 : kChunks - wide::kHalfK / 8;
     int dcount = 0;
-    bool ok_all = true;
     Sched sc, pv;
     bool pv_has_d = false;
     sc.init(sp, cstart);
-    for (int u = 0; ok_all; ++u) {
-      if (u >= 1) issue_rows(pv, group);  // the first chunk of tile u - 1, processed in (2)
-      // (1) move the D accumulator of tile u to this thread's shared-memory slot
-      bool cur_has_d = false;
-      if (sc.valid) {
-        bool dfull;
-        cur_has_d = sc.d_blocks(&dfull) > 0;
-        if (cur_has_d) {
-          const bool got = mbar_wait_bounded(dready_bar, static_cast<uint32_t>(dcount & 1), status,
-                                             abort_flag);
-          if (!__all_sync(0xffffffffu, got)) break;
-          tc_fence_after();
-          uint32_t *slot = dsc + (u & 1) * kDWords;
-#pragma unroll 1
-          for (int c = group; c < kChunks; c += wide::kGroups) {
-            uint32_t v[16];
-            tmem_ld_32x32b_x16(lane_base + (u & 1) * kN + 16 * c, v);
-            tmem_ld_wait();
+    int cur_missing = sc.valid ? sc.missing() : 0;  // of tile u
+    for (int u = 0;; ++u) {
+      // What tile u - 1 needs from global memory is asked for before D is moved and
+      // the accumulator waited for: its rows' factors, and its first chunk's words.
+      const int acc = (u - 1) & 1;
+      const uint32_t *slot = dsc + acc * kDWords;
+      Epi3<MODE> ep;
+      typename Epi3<MODE>::Fetch f[2] = {};  // chunks c and c + 1 in turn
+      float2 wk[2];                          // factors of SNPs k kf + lane and kf + 32 + lane
+      if (u >= 1) {
+        const int64_t kf = pv.k0() + wide::kHalfK * half;
+        ep.init(args, pv.j, pv.i0() + 64 * static_cast<int64_t>(rank) + 16 * quarter, kf, 8 * chunks,
+                quarter, half, lane, s_begin);
+        ep.fetch(f[0], args, 0, pv_has_d, slot, keep_pol);
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              const uint32_t d0 = static_cast<uint32_t>(__float2int_rn(__uint_as_float(v[2 * e])));
-              const uint32_t d1 = static_cast<uint32_t>(__float2int_rn(__uint_as_float(v[2 * e + 1])));
-              st_l2_keep(slot + (8 * c + e) * 128 + L, (d0 & 0xFFFFu) | (d1 << 16), keep_pol);
-            }
-          }
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(ddone_bar);  // the follower's is forwarded by warp 1
-          ++dcount;
+        for (int x = 0; x < 2; ++x) {
+          const int64_t k = kf + 32 * x + lane;
+          wk[x] = MODE == 1 && k < n_v ? __ldg(reinterpret_cast<const float2 *>(args.t.w) + k)
+                                       : make_float2(1.f, 1.f);
         }
       }
-      // (2) the tallies and CCC values of tile u - 1
+      const bool cur_has_d = sc.valid && cur_missing > 0;
+      // Moves the D accumulator of tile u to the warp's part of its slot.
+      auto move_d = [&]() {
+        const bool got = mbar_wait_bounded(dready_bar, static_cast<uint32_t>(dcount & 1), status,
+                                           abort_flag);
+        if (!__all_sync(0xffffffffu, got)) return false;
+        tc_fence_after();
+        uint32_t *to = dsc + (u & 1) * kDWords;
+#pragma unroll 2
+        for (int c = c_first; c < c_first + chunks; ++c) {
+          uint32_t v[16];
+          tmem_ld_32x32b_x16(lane_base + (u & 1) * kN + 16 * c, v);
+          tmem_ld_wait();
+#pragma unroll
+          for (int x = 0; x < 8; ++x) {
+            const int2 d = counts2(make_float2(__uint_as_float(v[2 * x]), __uint_as_float(v[2 * x + 1])));
+            st_l2_keep(to + (8 * c + x) * 128 + L, static_cast<uint32_t>(d.x | (d.y << 16)), keep_pol);
+          }
+        }
+        tc_fence_before();
+        __syncwarp();  // and every lane of the warp sees the words
+        if (lane == 0) mbar_arrive(ddone_bar);  // the follower's is forwarded by warp 1
+        ++dcount;
+        return true;
+      };
+      // D first: the tensor cores wait for the move (moving it after the previous
+      // tile's first chunk, where D is not ready yet, measured 5% slower).
+      if (cur_has_d && !move_d()) break;
+      // The tallies and CCC values of tile u - 1.
       if (u >= 1) {
         const int v = u - 1;
-        const int acc = v & 1;
         const bool got = mbar_wait_bounded(tfull_bar(acc), (v >> 1) & 1, status, abort_flag);
         if (!__all_sync(0xffffffffu, got)) break;
         tc_fence_after();
-        const int64_t j = pv.j;
-        const int64_t i = pv.i0() + 64 * static_cast<int64_t>(rank) + (L >> 1);
-        const bool row_ok = i < j;
-        const int64_t k_first = pv.k0();
-        const uint32_t t_x = lane_base + acc * kN;
-        const uint32_t *slot = dsc + acc * kDWords;
-        const int64_t span = n_v - 1 - j;
-        const int64_t base = slab_offset_dev(j, n_v) - s_begin + i * span - (j + 1);
-        const int64_t pbase = i * (2 * n_v - i - 1) / 2 - i - 1;  // pair (i, k) at pbase + k
-        float wi = 1.f, wj0 = 1.f, wj1 = 1.f;
-        if (want_ccc && persnp) {
-          if (row_ok) wi = __ldg(wv + 2 * i + a);
-          wj0 = __ldg(wv + 2 * j);
-          wj1 = __ldg(wv + 2 * j + 1);
-        }
-        constexpr int KC = 8;  // SNPs k per chunk (16 accumulator columns)
-        const int c_last = group + wide::kGroups * ((kChunks - 1 - group) / wide::kGroups);
-        for (int c = group; c < kChunks; c += wide::kGroups) {
-          const int kl = KC * c;  // first local SNP k of the chunk
-          const int64_t kc = k_first + kl;
-          uint32_t x[2 * KC];
-          tmem_ld_32x32b_x16(t_x + 2 * kl, x);
-          int2 r[KC];
-          float2 wk[KC];
-          uint32_t dd[KC];
-#pragma unroll
-          for (int kk = 0; kk < KC; ++kk) {
-            const int64_t k = kc + kk;
-            const bool ok = row_ok && k < n_v;
-            wk[kk] = (ok && want_ccc && persnp) ? __ldg(reinterpret_cast<const float2 *>(wv) + k)
-                                                : make_float2(1.f, 1.f);
-            dd[kk] = pv_has_d ? ld_l2_keep(slot + (kl + kk) * 128 + L, keep_pol) : 0u;
-          }
-          asm volatile("cp.async.wait_group 0;" ::: "memory");
-          __syncwarp();  // every lane's copies of the chunk have landed
-          const uint32_t rrow = rbuf + static_cast<uint32_t>((L >> 1) & 15) * wide::kRowStride +
-                                8u * static_cast<uint32_t>(a);
-#pragma unroll
-          for (int kk = 0; kk < KC; ++kk) {
-            const bool ok = row_ok && kc + kk < n_v &&
-                            CCC_IN_BOUNDS(pbase + kc + kk, n_v * (n_v - 1) / 2, args.t.status);
-            int2 v;
-            asm volatile("ld.shared.v2.s32 {%0, %1}, [%2];"
-                         : "=r"(v.x), "=r"(v.y)
-                         : "r"(rrow + 16u * kk)
-                         : "memory");
-            r[kk] = ok ? v : make_int2(0, 0);
-          }
-          // The buffer takes the next chunk's rows once every lane has read it.
-          __syncwarp();
-          if (c + wide::kGroups < kChunks) issue_rows(pv, c + wide::kGroups);
+        const uint32_t t_x = lane_base + acc * kN + 16 * c_first;
+        uint32_t x[16];
+        tmem_ld_32x32b_x16(t_x, x);
+        ep.products();
+        // Chunk c (h = its parity): its columns into the ring, the next chunk's loads, its lines.
+        auto chunk = [&](int c, int h) {
           tmem_ld_wait();
-          if (c == c_last) {
+          __syncwarp();  // the lines of chunk c - 1, which reach into chunk c - 2, have been read
+          ep.put(x, 128 * h, lane, ring);
+          if (MODE == 1 && (lane >> 3) == (c & 3))
+            *reinterpret_cast<float2 *>(wring + 64 * h + 8 * (lane & 7)) = c < 4 ? wk[0] : wk[1];
+          __syncwarp();
+          if (c + 1 < chunks) {
+            tmem_ld_32x32b_x16(t_x + 16 * (c + 1), x);
+          } else {  // every column is in the ring
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(tempty_bar(acc));  // the follower's is forwarded
           }
-#pragma unroll
-          for (int kk = 0; kk < KC; ++kk) {
-            const int64_t k = kc + kk;
-            const bool ok = row_ok && k < n_v && CCC_IN_BOUNDS(base + k, args.t.out_len, args.t.status);
-            const int32_t t0 = __float2int_rn(__uint_as_float(x[2 * kk]));
-            const int32_t t1 = __float2int_rn(__uint_as_float(x[2 * kk + 1]));
-            const int32_t d0 = static_cast<int32_t>(dd[kk] & 0xFFFFu);
-            const int32_t d1 = static_cast<int32_t>(dd[kk] >> 16);
-            const int32_t u0 = r[kk].x - d0, u1 = r[kk].y - d1;
-            // r^{a b c}: b0c0, b0c1, b1c0, b1c1
-            const int4 tv = make_int4(u0 + t0, u1 + t1, u0 - t0, u1 - t1);
-            const int64_t t = base + k;
-            if (ok) __stcs(tally_out + 2 * t + a, tv);
-            if (want_ccc) {
-              const int32_t own = tv.x + tv.y + tv.z + tv.w;  // sum over b, c (fixed a)
-              const int32_t n8 = own + __shfl_xor_sync(0xffffffffu, own, 1);
-              int32_t rb0 = 0, rb1 = 0, q0 = 0, q1 = 0;
-              if constexpr (!persnp) {
-                const int32_t b0 = tv.x + tv.y, b1 = tv.z + tv.w;
-                const int32_t c0 = tv.x + tv.z, c1 = tv.y + tv.w;
-                rb0 = b0 + __shfl_xor_sync(0xffffffffu, b0, 1);
-                rb1 = b1 + __shfl_xor_sync(0xffffffffu, b1, 1);
-                q0 = c0 + __shfl_xor_sync(0xffffffffu, c0, 1);
-                q1 = c1 + __shfl_xor_sync(0xffffffffu, c1, 1);
-              }
-              if (ok) {
-                const float dn = n8 == 0 ? 1.f : static_cast<float>(n8);
-                const float inv = rcp_count(dn);
-                const float2 f0 = make_float2(static_cast<float>(tv.x), static_cast<float>(tv.y));
-                const float2 f1 = make_float2(static_cast<float>(tv.z), static_cast<float>(tv.w));
-                float4 out;
-                if (persnp) {
-                  out = ccc3_persnp(f0, f1, inv, mul2(both(wi), make_float2(wj0, wj1)), wk[kk]);
-                } else {
-                  const float fi = joint_factor(static_cast<float>(own), dn, inv, gamma);
-                  const float2 fj = joint_factors(
-                      make_float2(static_cast<float>(rb0), static_cast<float>(rb1)), dn, inv, gamma);
-                  const float2 fk = joint_factors(
-                      make_float2(static_cast<float>(q0), static_cast<float>(q1)), dn, inv, gamma);
-                  out = ccc3_joint(f0, f1, dn, inv, fi, fj, fk);
-                }
-                __stcs(ccc_out + 2 * t + a, out);
-              }
-            }
-          }
+          ep.fetch(f[h ^ 1], args, 8 * (c + 1), pv_has_d, slot, keep_pol);
+          ep.line(args, 8 * c, 128 * h, f[h], ring, wring);
+        };
+#pragma unroll 1
+        for (int c = 0; c < chunks; c += 2) {
+          chunk(c, 0);
+          if (c + 1 < chunks) chunk(c + 1, 1);
         }
+        // The rows' last, partial lines.
+        if (chunks & 1)
+          ep.line(args, 8 * chunks, 128, f[1], ring, wring);
+        else
+          ep.line(args, 8 * chunks, 0, f[0], ring, wring);
       }
       if (!sc.valid) break;
       pv = sc;
       pv_has_d = cur_has_d;
       sc.advance(cstep);
+      if (sc.valid) cur_missing = sc.missing();
     }
-    // Copies still in flight (after a wait that gave up) land before the CTA exits.
-    asm volatile("cp.async.wait_all;" ::: "memory");
   }
 
   tc_fence_before();
@@ -1135,9 +1242,10 @@ __global__ void __launch_bounds__(wide::kThreads, 1) __cluster_dims__(2, 1, 1)
 // rows 2 s + x (x = allele) of every SNP s restricted to those individuals,
 // as e4m3 counts rho_s(x), zero-padded to a multiple of 128 columns:
 // cbuf[(slab * 2 n_v + 2 s + x) * kCap + column].
-// 128-thread CTAs with few registers: they fit beside a resident class-kernel
-// CTA (its warps leave under 2K registers on some SM sub-partitions), so the
-// next batch's preparation overlaps the current batch's tallies.
+// The class kernel's CTAs fill their SMs (all registers since its register
+// split, which gave more than the overlap did: prepared beside it, the next
+// batch slowed the class kernel by as much as it hid), so these run before it
+// and in its tail.
 constexpr int kPrepThreads = 128;
 
 // FP4: the compacted rows in e2m1 nibbles, 256 individuals in 128 bytes per row.
@@ -1391,10 +1499,7 @@ static int launch_wide_mode(const CUtensorMap &tmOp, const CUtensorMap &tmC, con
   if (dev_c < 0) return CCC_ECUDA;
   int &max_clusters = max_clusters_dev[dev_c];
   if (max_clusters == 0) {
-    if (cudaFuncSetAttribute(k_tally3_class_w<MODE, FP4>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(wide::kSmem)) != cudaSuccess)
-      return CCC_ECUDA;
+    if (!tcp::split_kernel_ready(k_tally3_class_w<MODE, FP4>, wide::kSmem)) return CCC_ECUDA;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeClusterDimension;
@@ -1455,6 +1560,8 @@ static int launch_tally3_class_w(const Tally3Args &a, const uint8_t *op, int64_t
   return launch_wide_mode<2, FP4>(tmOp, tmC, ca, sp, tiles, num_sms, s);
 }
 
+bool tc3_class_table16(int64_t n_f) { return n_f <= kWideMaxNf; }
+
 int64_t tc3_class_dscratch_bytes() {
   return static_cast<int64_t>(wide::kMaxCtas) * 2 * wide::kDWords * 4;
 }
@@ -1464,8 +1571,8 @@ int launch_tally3_class(const Tally3Args &a, const uint8_t *op, int64_t op_rows,
                         const int32_t *missing, uint32_t *dscratch, int64_t j0, int64_t j1,
                         int num_sms, cudaStream_t s, bool fp4) {
   if (j1 <= j0) return CCC_OK;
-  if (fp4 && !(a.n_f <= kWideMaxNf && dscratch != nullptr)) return CCC_EUNSUPPORTED;
-  if (a.n_f <= kWideMaxNf && dscratch != nullptr)
+  if (fp4 && !tc3_class_table16(a.n_f)) return CCC_EUNSUPPORTED;
+  if (tc3_class_table16(a.n_f))
     return fp4 ? launch_tally3_class_w<true>(a, op, op_rows, mrow0, kpad, rtab, cbuf, missing,
                                              dscratch, j0, j1, num_sms, s)
                : launch_tally3_class_w<false>(a, op, op_rows, mrow0, kpad, rtab, cbuf, missing,

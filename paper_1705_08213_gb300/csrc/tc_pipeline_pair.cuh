@@ -184,6 +184,17 @@ __device__ __forceinline__ void mma_commit_pair(uint32_t bar, uint16_t mask) {
       : "memory");
 }
 
+// Dynamic shared memory of a register-split kernel, and a check that it was
+// built with the registers that its warpgroups pass on: with fewer, the wait for
+// more would not end.
+template <class K>
+bool split_kernel_ready(K kernel, size_t smem) {
+  cudaFuncAttributes at;
+  return cudaFuncGetAttributes(&at, kernel) == cudaSuccess && at.numRegs == 168 &&
+         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              static_cast<int>(smem)) == cudaSuccess;
+}
+
 // For epilogues that load nothing early.
 struct NoEarly {};
 
