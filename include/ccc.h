@@ -137,7 +137,7 @@ typedef struct ccc_opts {
                              SNP tiles and long vectors.  0 = automatic (tensor cores: when the
                              triangle has at most half as many tiles as SM pairs and at least 32
                              128-byte K stages, n_f >= 4,096 with e4m3 and 8,192 with e2m1
-                             operands; popcount: fewer 64-SNP tiles than four per SM, at least
+                             operands; popcount: fewer 32-SNP tiles than four per SM, at least
                              4,096 individuals per part), 1 = off, n >= 2 = n parts (at most one
                              per K stage: n_f / 128 with e4m3, n_f / 256 with e2m1 operands,
                              n_f / 512 on the popcount path).  Same results;

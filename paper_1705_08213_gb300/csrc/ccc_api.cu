@@ -425,10 +425,10 @@ static int k_split_tiles(int requested, int64_t tiles, int64_t kpad, int sms) {
 }
 
 // K parts of a 2-way popcount call: opts->split when set (at most the 8-word
-// stages), else automatic: a triangle of fewer 64-SNP tiles than four per SM is
+// stages), else automatic: a triangle of fewer 32-SNP tiles than four per SM is
 // split into about 16 blocks per SM, each part keeping at least 64 words (4,096
-// individuals).  Measured on GB300, 512 SNPs (36 tiles) x 1,000,000: 9 parts
-// 12.3 ms, 18 parts 10.3, 36 parts 9.4, 72 parts 9.1.
+// individuals).  Measured on GB300, 512 SNPs (136 tiles) x 1,000,000: 3 parts
+// 6.81 ms, 9 parts 6.31, 18 parts (automatic) 5.93, 36 parts 5.76, 72 parts 5.71.
 static int popc_split(int requested, int64_t n_v, int64_t w64, int sms) {
   const int64_t stages = (w64 + 7) / 8;
   if (requested >= 1) return static_cast<int>(requested < stages ? requested : stages);

@@ -2,24 +2,35 @@
 // form of Sec. 3.1, where every 2-bit entry is handled by word-wide bitwise
 // operations and counted with a hardware population count.
 //
-// Each SNP is held as three bit planes per 64 entries (built by k_planes):
-// P1 = first copy of allele 1 (het or hom 1), P2 = second copy (hom 1),
-// M = present.  With rho_1 = P1 + P2 and rho_0 = 2M - rho_1:
-//   r11 = sum_q rho_1,i rho_1,j = |P1i&P1j| + |P1i&P2j| + |P2i&P1j| + |P2i&P2j|
-//   X   = sum_q rho_1,i m_j     = |P1i&Mj| + |P2i&Mj|
-//   Y   = sum_q m_i rho_1,j     = |Mi&P1j| + |Mi&P2j|
+// Each SNP is held as three bit planes per 64 entries (built by k_planes as
+// P1 = first copy of allele 1, P2 = second copy, M = present; a hom 1 entry has
+// both copies): H = P1 ^ P2 (het), A = P2 (hom 1), M.  With rho_1 = H + 2 A and
+// rho_0 = 2M - rho_1:
+//   r11 = sum_q rho_1,i rho_1,j = |Hi&Hj| + 2 (|Hi&Aj| + |Ai&Hj|) + 4 |Ai&Aj|
+//   X   = sum_q rho_1,i m_j     = |Hi&Mj| + 2 |Ai&Mj|
+//   Y   = sum_q m_i rho_1,j     = |Mi&Hj| + 2 |Mi&Aj|
 //   Z   = sum_q m_i m_j         = |Mi&Mj|
 //   r10 = 2X - r11,  r01 = 2Y - r11,  r00 = 4Z - 2X - 2Y + r11.
-// P2 is a subset of P1 (hom 1 implies a first copy), so of the four r11 terms
-// the last three take two population counts (see the inner loop): eight
-// POPC per 64 entries per pair; four accumulators per pair.
+// Hi&Aj and Ai&Hj exclude each other, so one population count takes both.
 //
-// Block tile: 64 x 64 SNPs of the upper triangle (J >= I), 256 threads, each
-// thread 4 x 4 pairs; the planes of both tiles are staged in shared memory 8
-// words (512 entries) at a time.  A K split (gridDim.y parts) gives each block
-// a range of words; since the four tallies are linear in the four sums, the
-// parts add their partial tallies into the zeroed output with integer
-// reductions, and the CCC values follow from the summed tallies (k_metric2).
+// The population count runs at a quarter of the rate of the bitwise operations
+// and is what bounds this form, so the products are not counted one by one:
+// carry-save adders (sum x^y^z, carry majority, two 3-input operations each)
+// add words of equal weight into a running word per weight, and only the
+// carries out of the highest running word are counted (Harley and Seal).  Per
+// four words and pair: 11 adders and 21 counts instead of 32 counts, which is
+// where counts (84 cycles of an SM per 32 pairs) and bitwise operations (about
+// 73) take about as long; three adders more for X, counted at weight 4 as r11
+// is, took the registers of the second block per SM (6.0 ms).  GB300, 4,096 x
+// 16,384: 8.23 -> 5.47 ms per call.
+//
+// Block tile: 32 x 32 SNPs of the upper triangle (J >= I), 256 threads, each
+// thread 2 x 2 pairs (running words and counts take 16 registers per pair); the planes
+// of both sides are staged in shared memory 8 words (512 entries) at a time.  A
+// K split (gridDim.y parts) gives each block a range of words; since the four
+// tallies are linear in the four sums, the parts add their partial tallies into
+// the zeroed output with integer reductions, and the CCC values follow from the
+// summed tallies (k_metric2).
 #include "ccc_dev.cuh"
 #include "ccc_launch.h"
 #include "ccc_metric.cuh"
@@ -27,7 +38,7 @@
 namespace ccc {
 namespace {
 
-constexpr int TS = 64;       // SNPs per tile side
+constexpr int TS = 32;       // SNPs per tile side
 constexpr int KC = 8;        // 64-entry words per stage
 constexpr int THREADS = 256;
 constexpr int LDS = TS + 1;  // padded row (u64) against bank conflicts
@@ -45,10 +56,11 @@ __device__ __forceinline__ void tile_coords(int64_t t, int64_t nB, int64_t &I, i
   J = r + (t - start(r));
 }
 
+// Planes H, A, M of 32 SNPs x KC words, 2 halves of 16 bytes per word.
 __device__ __forceinline__ void load_stage(const uint64_t *__restrict__ planes, int64_t w64,
                                            int64_t kend, int64_t n_v, int64_t snp0, int64_t k0,
                                            uint64_t (*s)[KC][LDS]) {
-  // 64 SNPs x KC words x 2 halves of 16 bytes.
+#pragma unroll
   for (int l = threadIdx.x; l < TS * KC * 2; l += THREADS) {
     const int half = l & 1;
     const int word = (l >> 1) % KC;
@@ -60,7 +72,7 @@ __device__ __forceinline__ void load_stage(const uint64_t *__restrict__ planes, 
     const uint64_t lo = (static_cast<uint64_t>(v.y) << 32) | v.x;
     const uint64_t hi = (static_cast<uint64_t>(v.w) << 32) | v.z;
     if (half == 0) {
-      s[0][word][snp] = lo;
+      s[0][word][snp] = lo ^ hi;
       s[1][word][snp] = hi;
     } else {
       s[2][word][snp] = lo;
@@ -68,7 +80,57 @@ __device__ __forceinline__ void load_stage(const uint64_t *__restrict__ planes, 
   }
 }
 
-__global__ void __launch_bounds__(THREADS)
+__device__ __forceinline__ uint64_t sum3(uint64_t a, uint64_t b, uint64_t c) { return a ^ b ^ c; }
+__device__ __forceinline__ uint32_t maj3(uint32_t a, uint32_t b, uint32_t c) {
+  uint32_t r;
+  asm("lop3.b32 %0, %1, %2, %3, 0xE8;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
+  return r;
+}
+
+// Carry-save adder: run takes the sum bits of run + a + b, the carries are returned.
+__device__ __forceinline__ uint64_t csa(uint64_t &run, uint64_t a, uint64_t b) {
+  const uint32_t lo = maj3(static_cast<uint32_t>(run), static_cast<uint32_t>(a), static_cast<uint32_t>(b));
+  const uint32_t hi = maj3(static_cast<uint32_t>(run >> 32), static_cast<uint32_t>(a >> 32),
+                           static_cast<uint32_t>(b >> 32));
+  run = sum3(run, a, b);
+  return (static_cast<uint64_t>(hi) << 32) | lo;
+}
+
+// One SNP's planes of a word.
+struct Word {
+  uint64_t h, a, m;
+};
+
+// The four sums of a pair: running words by weight, counts by weight.
+struct PairSums {
+  uint64_t r1 = 0, r2 = 0;          // r11, weights 1 and 2
+  uint64_t x1 = 0, y1 = 0, z1 = 0;  // X, Y, Z
+  uint32_t r4 = 0, x2 = 0, y2 = 0, z2 = 0;  // counts of weight 4, 2, 2, 2
+  uint64_t rc;  // r11's weight-2 carry of the first two words of four
+
+  // Words 2 half and 2 half + 1 of a group of four.
+  __device__ __forceinline__ void add(int half, const Word &i0, const Word &j0, const Word &i1,
+                                      const Word &j1) {
+    const uint64_t c = csa(r1, i0.h & j0.h, i1.h & j1.h);
+    r4 += __popcll(csa(r2, (i0.h & j0.a) | (i0.a & j0.h), (i1.h & j1.a) | (i1.a & j1.h)));
+    r4 += __popcll(i0.a & j0.a) + __popcll(i1.a & j1.a);
+    if (half == 0)
+      rc = c;
+    else
+      r4 += __popcll(csa(r2, rc, c));
+    x2 += __popcll(csa(x1, i0.h & j0.m, i1.h & j1.m));
+    x2 += __popcll(i0.a & j0.m) + __popcll(i1.a & j1.m);
+    y2 += __popcll(csa(y1, i0.m & j0.h, i1.m & j1.h));
+    y2 += __popcll(i0.m & j0.a) + __popcll(i1.m & j1.a);
+    z2 += __popcll(csa(z1, i0.m & j0.m, i1.m & j1.m));
+  }
+  __device__ __forceinline__ int32_t r11() const { return __popcll(r1) + 2 * __popcll(r2) + 4 * r4; }
+  __device__ __forceinline__ int32_t x() const { return __popcll(x1) + 2 * x2; }
+  __device__ __forceinline__ int32_t y() const { return __popcll(y1) + 2 * y2; }
+  __device__ __forceinline__ int32_t z() const { return __popcll(z1) + 2 * z2; }
+};
+
+__global__ void __launch_bounds__(THREADS, 2)
     k_tally2_popc(const uint64_t *__restrict__ planes, int64_t w64, const Tally2Args args,
                   int64_t nB, int64_t t0, int64_t part_words) {
   __shared__ uint64_t sI[3][KC][LDS];
@@ -78,13 +140,7 @@ __global__ void __launch_bounds__(THREADS)
   const int64_t n_v = args.n_v;
   const int tx = threadIdx.x & 15;
   const int ty = threadIdx.x >> 4;
-  uint32_t acc[4][4][4];
-#pragma unroll
-  for (int x = 0; x < 4; ++x)
-#pragma unroll
-    for (int y = 0; y < 4; ++y)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) acc[x][y][c] = 0u;
+  PairSums acc[2][2];
 
   const int64_t kbeg = static_cast<int64_t>(blockIdx.y) * part_words;
   const int64_t kend = kbeg + part_words < w64 ? kbeg + part_words : w64;
@@ -92,39 +148,27 @@ __global__ void __launch_bounds__(THREADS)
     load_stage(planes, w64, kend, n_v, I * TS, k0, sI);
     load_stage(planes, w64, kend, n_v, J * TS, k0, sJ);
     __syncthreads();
-#pragma unroll 4
-    for (int k = 0; k < KC; ++k) {
-      uint64_t a1[4], a2[4], am[4], b1[4], b2[4], bm[4];
 #pragma unroll
-      for (int x = 0; x < 4; ++x) {
-        a1[x] = sI[0][k][ty + 16 * x];
-        a2[x] = sI[1][k][ty + 16 * x];
-        am[x] = sI[2][k][ty + 16 * x];
-      }
+    for (int k = 0; k < KC; k += 2) {
+      Word wi[2][2], wj[2][2];  // [SNP][word]
 #pragma unroll
-      for (int y = 0; y < 4; ++y) {
-        b1[y] = sJ[0][k][tx + 16 * y];
-        b2[y] = sJ[1][k][tx + 16 * y];
-        bm[y] = sJ[2][k][tx + 16 * y];
-      }
+      for (int x = 0; x < 2; ++x)
 #pragma unroll
-      for (int x = 0; x < 4; ++x)
-#pragma unroll
-        for (int y = 0; y < 4; ++y) {
-          // P2 is a subset of P1, so (P1i & P2j) & (P2i & P1j) = P2i & P2j and
-          // |P1i&P2j| + |P2i&P1j| + |P2i&P2j| = |p ^ q| + 3 |p & q|.
-          const uint64_t p = a1[x] & b2[y], q = a2[x] & b1[y];
-          acc[x][y][0] += __popcll(a1[x] & b1[y]) + __popcll(p ^ q) + 3 * __popcll(p & q);
-          acc[x][y][1] += __popcll(a1[x] & bm[y]) + __popcll(a2[x] & bm[y]);
-          acc[x][y][2] += __popcll(am[x] & b1[y]) + __popcll(am[x] & b2[y]);
-          acc[x][y][3] += __popcll(am[x] & bm[y]);
+        for (int w = 0; w < 2; ++w) {
+          wi[x][w] = Word{sI[0][k + w][ty + 16 * x], sI[1][k + w][ty + 16 * x], sI[2][k + w][ty + 16 * x]};
+          wj[x][w] = Word{sJ[0][k + w][tx + 16 * x], sJ[1][k + w][tx + 16 * x], sJ[2][k + w][tx + 16 * x]};
         }
+#pragma unroll
+      for (int x = 0; x < 2; ++x)
+#pragma unroll
+        for (int y = 0; y < 2; ++y)
+          acc[x][y].add((k >> 1) & 1, wi[x][0], wj[y][0], wi[x][1], wj[y][1]);
     }
     __syncthreads();
   }
 
 #pragma unroll
-  for (int x = 0; x < 4; ++x) {
+  for (int x = 0; x < 2; ++x) {
     const int64_t i = I * TS + ty + 16 * x;
     if (i >= n_v || i < args.i_begin || i >= args.i_end) continue;
     const bool filter = args.hits != nullptr;
@@ -137,13 +181,10 @@ __global__ void __launch_bounds__(THREADS)
     }
     const int64_t row_base = i * (2 * n_v - i - 1) / 2 - i - 1 - args.pair0;
 #pragma unroll
-    for (int y = 0; y < 4; ++y) {
+    for (int y = 0; y < 2; ++y) {
       const int64_t j = J * TS + tx + 16 * y;
       if (!(i < j && j < n_v)) continue;
-      const int32_t r11 = static_cast<int32_t>(acc[x][y][0]);
-      const int32_t X = static_cast<int32_t>(acc[x][y][1]);
-      const int32_t Y = static_cast<int32_t>(acc[x][y][2]);
-      const int32_t Z = static_cast<int32_t>(acc[x][y][3]);
+      const int32_t r11 = acc[x][y].r11(), X = acc[x][y].x(), Y = acc[x][y].y(), Z = acc[x][y].z();
       const int32_t r10 = 2 * X - r11;
       const int32_t r01 = 2 * Y - r11;
       const int32_t r00 = 4 * Z - 2 * X - 2 * Y + r11;
