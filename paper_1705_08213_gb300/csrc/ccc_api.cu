@@ -370,10 +370,10 @@ static int launch_tally2_tc_auto(const Tally2Args &a, const ccc_opts *o, const u
 // (from the same read of the codes for e2m1 rows and for K-block-major rows).
 static int unpack_2way(const ccc_panel *p, const ccc_opts *o, uint8_t *op, int64_t kpad,
                        int64_t rows_pad, cudaStream_t s, int64_t blocked_rows = 0,
-                       float *w = nullptr) {
+                       float *w = nullptr, int32_t *counts = nullptr) {
   if (fp4_2way(o))
     return launch_unpack_e2m1(p->geno, p->n_f, p->n_v, p->ld, op, kpad, rows_pad / 2, s,
-                              blocked_rows, w, o->gamma);
+                              blocked_rows, w, o->gamma, counts);
   if (blocked_rows > 0)
     return launch_unpack_blocked(p->geno, p->n_f, p->n_v, p->ld, op, kpad, rows_pad / 2,
                                  blocked_rows, false, w, o->gamma, s);
@@ -499,6 +499,9 @@ static int run_2way(const ccc_panel *p, int32_t *tally, float *out_ccc, const cc
   a.n_v = p->n_v;
   a.n_f = p->n_f;
   a.w = w;
+  // The FP4 thresholded kernel also takes the counts n_i (see Epi2Rect).
+  int32_t *counts = filter != nullptr && want_w && fp4 ? at<int32_t>(o, L.counts) : nullptr;
+  a.counts = counts;
   a.tally = tally;
   a.ccc = out_ccc;
   a.status = at<int32_t>(o, L.status);
@@ -520,7 +523,7 @@ static int run_2way(const ccc_panel *p, int32_t *tally, float *out_ccc, const cc
     // The K-split kernel reads its operand K-block-major.
     if (!packed)
       CCC_TRY(unpack_2way(p, o, op, L.kpad, L.rows_pad, s, split > 1 ? L.rows_pad : 0,
-                          want_w ? w : nullptr));
+                          want_w ? w : nullptr, counts));
     if (split > 1) {
       // Partial tallies of the K parts are summed into the zeroed output; the
       // CCC values follow from the complete tallies.

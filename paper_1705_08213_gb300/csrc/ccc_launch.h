@@ -67,10 +67,10 @@ int launch_unpack_e4m3(const uint64_t *geno, int64_t n_f, int64_t n_v, int64_t l
 // The same with e2m1 (FP4) counts, two entries per byte: rows of kpad / 2
 // bytes (kpad a multiple of 256); blocked: [kpad / 256][blocked_rows][128].
 // w != null: also the per-SNP factors of launch_allele_counts (w[n_v][2],
-// 1 - gamma f_i(a)) from the same read of the codes.
+// 1 - gamma f_i(a)) and, if counts is set, its counts, from the same read of the codes.
 int launch_unpack_e2m1(const uint64_t *geno, int64_t n_f, int64_t n_v, int64_t ld, uint8_t *op,
                        int64_t kpad, int64_t snps_pad, cudaStream_t s, int64_t blocked_rows = 0,
-                       float *w = nullptr, double gamma = 0.0);
+                       float *w = nullptr, double gamma = 0.0, int32_t *counts = nullptr);
 int launch_planes(const uint64_t *geno, int64_t n_f, int64_t n_v, int64_t ld, uint64_t *planes,
                   int64_t w64, cudaStream_t s);
 
@@ -93,6 +93,8 @@ struct Tally2Args {
   int64_t n_v;
   int64_t n_f;
   const float *w;   // [n_v][2] per-SNP factors 1 - gamma f_i(a) (PERSNP), or null
+  // [n_v][3] allele counts; the third, n_i, with w for thresholded PERSNP output.
+  const int32_t *counts = nullptr;
   int32_t *tally;   // [npairs][4]
   float *ccc;       // [npairs][4] or null (tallies only)
   int32_t *status;  // workspace status word

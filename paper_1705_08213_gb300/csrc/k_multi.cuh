@@ -84,7 +84,7 @@ struct EpiMultiT {
   // The warps of column half h (c0 = h NC) take the chunks of 32 columns
   // [h NBQ / 2, (h + 1) NBQ / 2); chunk c is B quarter NBQ J + c.
   template <int NC>
-  __device__ __forceinline__ static tcp::NoEarly early(const Params &, const Sched &, int, int, int, int) {
+  __device__ __forceinline__ static tcp::NoEarly early(const Params &, const Sched &, bool, int, int, int, int) {
     return {};
   }
   template <int NC, bool PRELOAD = false>
@@ -187,7 +187,7 @@ struct EpiMultiSplit {
   static constexpr int STAGE_BYTES_PER_WARP = 0;
 
   template <int NC>
-  __device__ __forceinline__ static tcp::NoEarly early(const Params &, const SplitSchedPair &, int, int, int, int) {
+  __device__ __forceinline__ static tcp::NoEarly early(const Params &, const SplitSchedPair &, bool, int, int, int, int) {
     return {};
   }
   template <int NC, bool PRELOAD = false>

@@ -215,7 +215,8 @@ __global__ void k_unpack_e2m1(const uint64_t *__restrict__ geno, int64_t n_f, in
 __global__ void __launch_bounds__(128) k_unpack_e2m1_w(const uint64_t *__restrict__ geno,
                                                       int64_t n_f, int64_t n_v, int64_t ld,
                                                       uint8_t *__restrict__ op, int64_t kpad,
-                                                      float *__restrict__ w, double gamma) {
+                                                      float *__restrict__ w, double gamma,
+                                                      int32_t *__restrict__ counts) {
   __shared__ long long part[4][2];
   const int64_t i = blockIdx.x;
   const int64_t wpr = kpad / 32;
@@ -275,6 +276,11 @@ __global__ void __launch_bounds__(128) k_unpack_e2m1_w(const uint64_t *__restric
     const double f1 = n > 0 ? static_cast<double>(s1) / (2.0 * static_cast<double>(n)) : 0.0;
     w[2 * i + 0] = static_cast<float>(1.0 - gamma * f0);
     w[2 * i + 1] = static_cast<float>(1.0 - gamma * f1);
+    if (counts) {
+      counts[3 * i + 0] = static_cast<int32_t>(s0);
+      counts[3 * i + 1] = static_cast<int32_t>(s1);
+      counts[3 * i + 2] = static_cast<int32_t>(n);
+    }
   }
 }
 
@@ -515,7 +521,7 @@ int launch_unpack_e4m3(const uint64_t *geno, int64_t n_f, int64_t n_v, int64_t l
 
 int launch_unpack_e2m1(const uint64_t *geno, int64_t n_f, int64_t n_v, int64_t ld, uint8_t *op,
                        int64_t kpad, int64_t snps_pad, cudaStream_t s, int64_t blocked_rows,
-                       float *w, double gamma) {
+                       float *w, double gamma, int32_t *counts) {
   if (kpad % 256 != 0) return CCC_EINVAL;
   if (blocked_rows != 0)
     return launch_unpack_blocked(geno, n_f, n_v, ld, op, kpad, snps_pad, blocked_rows, true, w,
@@ -526,11 +532,11 @@ int launch_unpack_e2m1(const uint64_t *geno, int64_t n_f, int64_t n_v, int64_t l
   if (w != nullptr && snps_pad >= 152 * 8) {
     if (snps_pad < n_v) return CCC_EINVAL;
     k_unpack_e2m1_w<<<static_cast<unsigned>(snps_pad), 128, 0, s>>>(geno, n_f, n_v, ld, op, kpad,
-                                                                     w, gamma);
+                                                                     w, gamma, counts);
     return note_launch();
   }
   if (w != nullptr) {
-    const int rc = launch_allele_counts(geno, n_f, n_v, ld, nullptr, w, gamma, s);
+    const int rc = launch_allele_counts(geno, n_f, n_v, ld, counts, w, gamma, s);
     if (rc != CCC_OK) return rc;
   }
   const int threads = 256;

@@ -202,9 +202,9 @@ struct NoEarly {};
 // give the first row of the tile (the CTA adds 128 r); map_index() selects the
 // tile's tensor map in tm[]; the tile's K stages are k_begin() ..
 // k_begin() + k_blocks(nkb) - 1.
-// Epi: template <int NC> static T early(const Params&, const Sched&, int rank,
-//        int quarter, int lane, int c0): what the tile's epilogue needs from
-//        global memory, loaded before the accumulator is waited for;
+// Epi: template <int NC> static T early(const Params&, const Sched&, bool tile,
+//        int rank, int quarter, int lane, int c0): what the tile's epilogue needs
+//        from global memory, loaded ahead of it (tile: there is one);
 //      template <int NC> static void tile(const Params&, const Sched&, int rank,
 //        int quarter, int lane, uint32_t t_base, uint32_t release_cluster_bar,
 //        int c0, float *stage, const T&, bool more); the release arrives at a
@@ -416,13 +416,22 @@ __device__ __forceinline__ void persistent_gemm_pair(const CUtensorMap *tm,
     constexpr int NC = tc::Epilogue<EW>::CHUNKS_PER_WARP;
     const int c0 = half * NC;
     int lt = 0;
+    // What a tile needs from global memory is loaded before its accumulator is
+    // waited for; with two accumulators, where the epilogue may be the later side
+    // and the wait short, during the tile before.
+    auto load = [&](const Sched &t, bool tile) {
+      return Epi::template early<NC>(ep, t, tile, static_cast<int>(rank), quarter, lane, c0);
+    };
     Sched sc, next;
-    for (sc.init(sp, cstart); sc.valid; sc = next, ++lt) {
+    sc.init(sp, cstart);
+    auto ahead = load(sc, NACC == 2 && sc.valid);
+    for (; sc.valid; sc = next, ++lt) {
       next = sc;
       next.advance(cstep);
+      const auto early = NACC == 1 ? load(sc, true) : ahead;
+      if constexpr (NACC == 2) ahead = load(next, next.valid);
       const int acc = NACC == 1 ? 0 : (lt & 1);
       const uint32_t acc_phase = NACC == 1 ? (lt & 1) : ((lt >> 1) & 1);
-      const auto early = Epi::template early<NC>(ep, sc, static_cast<int>(rank), quarter, lane, c0);
       const bool ok = mbar_wait_bounded(tfull_bar(acc), acc_phase, status, abort_flag);
       if (!__all_sync(0xffffffffu, ok)) break;
       tc_fence_after();
@@ -696,7 +705,8 @@ __device__ __forceinline__ void persistent_gemm_pair_packed(const CUtensorMap *t
     for (sc.init(sp, cstart); sc.valid; sc.advance(cstep), ++lt) {
       const int acc = lt & 1;
       const uint32_t acc_phase = (lt >> 1) & 1;
-      const auto early = Epi::template early<NC>(ep, sc, static_cast<int>(rank), quarter, lane, c0);
+      const auto early =
+          Epi::template early<NC>(ep, sc, true, static_cast<int>(rank), quarter, lane, c0);
       const bool ok = mbar_wait_bounded(tfull_bar(acc), acc_phase, status, abort_flag);
       if (!__all_sync(0xffffffffu, ok)) break;
       tc_fence_after();
