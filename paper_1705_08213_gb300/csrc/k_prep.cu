@@ -152,15 +152,50 @@ __global__ void k_unpack_e4m3(const uint64_t *__restrict__ geno, int64_t n_f, in
   *reinterpret_cast<uint4 *>(d1) = make_uint4(r1[0], r1[1], r1[2], r1[3]);
 }
 
-// Spread the sixteen 2-bit fields of x into the low two bits of sixteen 4-bit
-// fields (field q of x -> bits 4q, 4q + 1 of the result).
-__device__ __forceinline__ uint64_t spread_2to4(uint32_t x32) {
-  uint64_t x = x32;
-  x = (x | (x << 16)) & 0x0000FFFF0000FFFFull;
-  x = (x | (x << 8)) & 0x00FF00FF00FF00FFull;
-  x = (x | (x << 4)) & 0x0F0F0F0F0F0F0F0Full;
-  x = (x | (x << 2)) & 0x3333333333333333ull;
-  return x;
+// The e2m1 nibbles of eight 2-bit codes (the low 16 bits of x): the codes are
+// spread to nibbles once and both rows formed there, l = low, h = high code bit:
+// rho(1) = 1 for l & ~h (0x2) and 2 for l & h (0x4), rho(0) = 1 for l & ~h and 2
+// for neither; both are 0 for the missing code (h & ~l).  Spreading the two
+// rows' counts apart took about twice the instructions, which bounded the
+// unpack of long vectors (512 x 1,000,000: 149 -> 118 us, 5.4 TB/s, with 4 loads
+// in flight per thread and one population count less per word).
+__device__ __forceinline__ void nibbles8(uint32_t x, uint32_t &n0, uint32_t &n1) {
+  x &= 0xFFFFu;
+  x = (x | (x << 8)) & 0x00FF00FFu;
+  x = (x | (x << 4)) & 0x0F0F0F0Fu;
+  x = (x | (x << 2)) & 0x33333333u;
+  const uint32_t h = x >> 1;
+  const uint32_t het = (x & ~h & 0x11111111u) << 1;
+  n0 = het | ((~(x | h) & 0x11111111u) << 2);
+  n1 = het | ((x & h & 0x11111111u) << 2);
+}
+
+// The 16 bytes of both operand rows of a packed word (32 entries).
+__device__ __forceinline__ void nibbles32(uint64_t v, uint4 &q0, uint4 &q1) {
+  const uint32_t lo = static_cast<uint32_t>(v), hi = static_cast<uint32_t>(v >> 32);
+  nibbles8(lo, q0.x, q1.x);
+  nibbles8(lo >> 16, q0.y, q1.y);
+  nibbles8(hi, q0.z, q1.z);
+  nibbles8(hi >> 16, q0.w, q1.w);
+}
+
+constexpr uint64_t kAllMissing = 0xAAAAAAAAAAAAAAAAull;
+
+// Word k of a row with the entries past n_f marked missing.
+__device__ __forceinline__ uint64_t mask_word(uint64_t raw, int64_t k, int64_t n_f) {
+  if ((k + 1) * 32 <= n_f) return raw;
+  if (k * 32 >= n_f) return kAllMissing;
+  const uint64_t valid = valid_even_mask(k, n_f);
+  const uint64_t vm = valid | (valid << 1);
+  return (raw & vm) | (kAllMissing & ~vm);
+}
+
+// Adds a masked word's present entries and allele-1 copies: rho(1) = l + (l & h),
+// counted in one word.
+__device__ __forceinline__ void count_word(uint64_t v, int32_t &n, int32_t &s1) {
+  const uint64_t l = v & kEven, h = (v >> 1) & kEven;
+  n += 32 - __popcll(h & ~l);
+  s1 += __popcll(l | ((l & h) << 1));
 }
 
 // FP4 (e2m1) operand rows: as k_unpack_e4m3, with each count 0, 1, 2 stored as
@@ -179,32 +214,13 @@ __global__ void k_unpack_e2m1(const uint64_t *__restrict__ geno, int64_t n_f, in
   if (t >= wpr * snps_pad) return;
   const int64_t i = t / wpr;
   const int64_t k = t - i * wpr;
-  uint64_t v = 0xAAAAAAAAAAAAAAAAull;  // all entries "missing" -> zero operands
-  if (i < n_v && k * 32 < n_f) {
-    const uint64_t valid = valid_even_mask(k, n_f);
-    const uint64_t vm = valid | (valid << 1);
-    v = (__ldg(geno + i * ld + k) & vm) | (0xAAAAAAAAAAAAAAAAull & ~vm);
-  }
-  uint64_t n0[2], n1[2];
-#pragma unroll
-  for (int half = 0; half < 2; ++half) {
-    const uint32_t x = static_cast<uint32_t>(v >> (32 * half));
-    const uint32_t l = x & 0x55555555u;
-    const uint32_t h = (x >> 1) & 0x55555555u;
-    const uint32_t nh = ~h & 0x55555555u;
-    const uint32_t rho1 = l + (l & h);         // 2-bit fields 0, 1, 2
-    const uint32_t rho0 = (nh << 1) - (l & nh);  // no borrow between fields
-    n0[half] = spread_2to4(rho0) << 1;
-    n1[half] = spread_2to4(rho1) << 1;
-  }
+  const uint64_t v =
+      i < n_v && k * 32 < n_f ? mask_word(__ldg(geno + i * ld + k), k, n_f) : kAllMissing;
+  uint4 q0, q1;
+  nibbles32(v, q0, q1);
   uint8_t *d0 = op + (2 * i) * (kpad / 2) + k * 16;  // row-major [row][kpad / 2]
-  uint8_t *d1 = d0 + kpad / 2;
-  *reinterpret_cast<uint4 *>(d0) =
-      make_uint4(static_cast<uint32_t>(n0[0]), static_cast<uint32_t>(n0[0] >> 32),
-                 static_cast<uint32_t>(n0[1]), static_cast<uint32_t>(n0[1] >> 32));
-  *reinterpret_cast<uint4 *>(d1) =
-      make_uint4(static_cast<uint32_t>(n1[0]), static_cast<uint32_t>(n1[0] >> 32),
-                 static_cast<uint32_t>(n1[1]), static_cast<uint32_t>(n1[1] >> 32));
+  *reinterpret_cast<uint4 *>(d0) = q0;
+  *reinterpret_cast<uint4 *>(d0 + kpad / 2) = q1;
 }
 
 // k_unpack_e2m1 with the per-SNP factors w = 1 - gamma f_i(a) of
@@ -217,43 +233,31 @@ __global__ void __launch_bounds__(128) k_unpack_e2m1_w(const uint64_t *__restric
                                                       uint8_t *__restrict__ op, int64_t kpad,
                                                       float *__restrict__ w, double gamma,
                                                       int32_t *__restrict__ counts) {
-  __shared__ long long part[4][2];
+  __shared__ int32_t part[4][2];
   const int64_t i = blockIdx.x;
   const int64_t wpr = kpad / 32;
   const bool snp = i < n_v;
-  int64_t n = 0, s1 = 0;
-  for (int64_t k = threadIdx.x; k < wpr; k += 128) {
-    uint64_t v = 0xAAAAAAAAAAAAAAAAull;  // all entries "missing" -> zero operands
-    if (snp && k * 32 < n_f) {
-      const uint64_t raw = __ldg(geno + i * ld + k);
-      const uint64_t valid = valid_even_mask(k, n_f);
-      const uint64_t l = raw & valid;
-      const uint64_t h = (raw >> 1) & valid;
-      n += __popcll(valid & ~(h & ~l));
-      s1 += __popcll(l) + __popcll(h & l);
-      const uint64_t vm = valid | (valid << 1);
-      v = (raw & vm) | (0xAAAAAAAAAAAAAAAAull & ~vm);
-    }
-    uint64_t n0[2], n1[2];
+  int32_t n = 0, s1 = 0;
+  // Two words per thread in flight.
+  for (int64_t k0 = threadIdx.x; k0 < wpr; k0 += 256) {
+    uint64_t v[2];
 #pragma unroll
-    for (int half = 0; half < 2; ++half) {
-      const uint32_t x = static_cast<uint32_t>(v >> (32 * half));
-      const uint32_t l = x & 0x55555555u;
-      const uint32_t h = (x >> 1) & 0x55555555u;
-      const uint32_t nh = ~h & 0x55555555u;
-      const uint32_t rho1 = l + (l & h);
-      const uint32_t rho0 = (nh << 1) - (l & nh);
-      n0[half] = spread_2to4(rho0) << 1;
-      n1[half] = spread_2to4(rho1) << 1;
+    for (int u = 0; u < 2; ++u) {
+      const int64_t k = k0 + 128 * u;
+      v[u] = snp && k * 32 < n_f ? __ldg(geno + i * ld + k) : kAllMissing;
     }
-    uint8_t *d0 = op + (2 * i) * (kpad / 2) + k * 16;
-    uint8_t *d1 = d0 + kpad / 2;
-    *reinterpret_cast<uint4 *>(d0) =
-        make_uint4(static_cast<uint32_t>(n0[0]), static_cast<uint32_t>(n0[0] >> 32),
-                   static_cast<uint32_t>(n0[1]), static_cast<uint32_t>(n0[1] >> 32));
-    *reinterpret_cast<uint4 *>(d1) =
-        make_uint4(static_cast<uint32_t>(n1[0]), static_cast<uint32_t>(n1[0] >> 32),
-                   static_cast<uint32_t>(n1[1]), static_cast<uint32_t>(n1[1] >> 32));
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int64_t k = k0 + 128 * u;
+      if (k >= wpr) break;
+      v[u] = mask_word(v[u], k, n_f);
+      count_word(v[u], n, s1);
+      uint4 q0, q1;
+      nibbles32(v[u], q0, q1);
+      uint8_t *d0 = op + (2 * i) * (kpad / 2) + k * 16;
+      *reinterpret_cast<uint4 *>(d0) = q0;
+      *reinterpret_cast<uint4 *>(d0 + kpad / 2) = q1;
+    }
   }
   if (!snp) return;  // the whole block: i is uniform
 #pragma unroll
@@ -309,56 +313,42 @@ __global__ void __launch_bounds__(256) k_unpack_blocked(const uint64_t *__restri
   uint8_t *base = op + 2 * i * 128 + sub * 16;
   const int64_t kb_stride = blocked_rows * 128;
   int32_t n = 0, s1 = 0;
-#pragma unroll 4
-  for (int64_t kb = kb0; kb < kb1; ++kb) {
-    const int64_t c = kb * 8 + sub;      // 16-byte piece of the row pair
-    const int64_t k = FP4 ? c : c >> 1;  // packed word
-    uint64_t v = 0xAAAAAAAAAAAAAAAAull;  // all entries "missing" -> zero operands
-    if (snp && k * 32 < n_f) {
-      const uint64_t valid = valid_even_mask(k, n_f);
-      const uint64_t vm = valid | (valid << 1);
-      v = (__ldg(row + k) & vm) | (0xAAAAAAAAAAAAAAAAull & ~vm);
-    }
-    if constexpr (COUNT) {
-      // Present entries (not h & ~l) and rho(1) = l + (l & h) of this thread's
-      // entries: the whole word (e2m1) or its half (e4m3); padding reads as missing.
-      const uint64_t x = FP4 ? v : (v >> (32 * (sub & 1))) & 0xFFFFFFFFull;
-      const uint64_t even = FP4 ? kEven : 0x55555555ull;
-      const uint64_t l = x & even, h = (x >> 1) & even;
-      n += __popcll(even & ~(h & ~l));
-      s1 += __popcll(l) + __popcll(h & l);
-    }
-    uint4 q0, q1;
-    if constexpr (FP4) {
-      uint64_t n0[2], n1[2];
+  constexpr int U = 4;  // K blocks whose loads are in flight
+  for (int64_t kb = kb0; kb < kb1; kb += U) {
+    uint64_t v[U];
 #pragma unroll
-      for (int half = 0; half < 2; ++half) {
-        const uint32_t x = static_cast<uint32_t>(v >> (32 * half));
-        const uint32_t l = x & 0x55555555u;
-        const uint32_t h = (x >> 1) & 0x55555555u;
-        const uint32_t nh = ~h & 0x55555555u;
-        n0[half] = spread_2to4((nh << 1) - (l & nh)) << 1;
-        n1[half] = spread_2to4(l + (l & h)) << 1;
-      }
-      q0 = make_uint4(static_cast<uint32_t>(n0[0]), static_cast<uint32_t>(n0[0] >> 32),
-                      static_cast<uint32_t>(n0[1]), static_cast<uint32_t>(n0[1] >> 32));
-      q1 = make_uint4(static_cast<uint32_t>(n1[0]), static_cast<uint32_t>(n1[0] >> 32),
-                      static_cast<uint32_t>(n1[1]), static_cast<uint32_t>(n1[1] >> 32));
-    } else {
-      const uint32_t h = static_cast<uint32_t>(v >> (32 * (sub & 1)));
-      uint32_t r0[4], r1[4];
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const uint32_t sel = code_nibbles((h >> (8 * b)) & 0xFFu);
-        r0[b] = __byte_perm(kRho0E4M3, 0u, sel);
-        r1[b] = __byte_perm(kRho1E4M3, 0u, sel);
-      }
-      q0 = make_uint4(r0[0], r0[1], r0[2], r0[3]);
-      q1 = make_uint4(r1[0], r1[1], r1[2], r1[3]);
+    for (int u = 0; u < U; ++u) {
+      const int64_t c = (kb + u) * 8 + sub;  // 16-byte piece of the row pair
+      const int64_t k = FP4 ? c : c >> 1;    // packed word
+      v[u] = snp && kb + u < kb1 && k * 32 < n_f ? __ldg(row + k) : kAllMissing;
     }
-    uint8_t *d0 = base + kb * kb_stride;
-    *reinterpret_cast<uint4 *>(d0) = q0;
-    *reinterpret_cast<uint4 *>(d0 + 128) = q1;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (kb + u >= kb1) break;
+      const int64_t c = (kb + u) * 8 + sub;
+      v[u] = mask_word(v[u], FP4 ? c : c >> 1, n_f);
+      uint4 q0, q1;
+      if constexpr (FP4) {
+        if (COUNT) count_word(v[u], n, s1);
+        nibbles32(v[u], q0, q1);
+      } else {
+        // This thread's half of the word (the other half counts as missing).
+        const uint32_t h = static_cast<uint32_t>(v[u] >> (32 * (sub & 1)));
+        if (COUNT) count_word(h | (kAllMissing << 32), n, s1);
+        uint32_t r0[4], r1[4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          const uint32_t sel = code_nibbles((h >> (8 * b)) & 0xFFu);
+          r0[b] = __byte_perm(kRho0E4M3, 0u, sel);
+          r1[b] = __byte_perm(kRho1E4M3, 0u, sel);
+        }
+        q0 = make_uint4(r0[0], r0[1], r0[2], r0[3]);
+        q1 = make_uint4(r1[0], r1[1], r1[2], r1[3]);
+      }
+      uint8_t *d0 = base + (kb + u) * kb_stride;
+      *reinterpret_cast<uint4 *>(d0) = q0;
+      *reinterpret_cast<uint4 *>(d0 + 128) = q1;
+    }
   }
   if constexpr (COUNT) {
     // The 8 threads of a SNP are 8 aligned lanes of one warp.
@@ -475,10 +465,10 @@ int launch_unpack_blocked(const uint64_t *geno, int64_t n_f, int64_t n_v, int64_
     return CCC_EINVAL;
   const int64_t nkb = kpad / kblock;
   if (snps_pad < 1 || nkb < 1) return CCC_OK;
-  // 32-SNP blocks times K ranges, about 16 blocks per SM in all.
+  // 32-SNP blocks times K ranges, about 32 blocks per SM in all.
   const int64_t gx = snps_pad / 32;
   if (gx > 0x7FFFFFFF) return CCC_EINVAL;
-  int64_t gy = (152 * 16 + gx - 1) / gx;
+  int64_t gy = (152 * 32 + gx - 1) / gx;
   if (gy > nkb) gy = nkb;
   if (gy > 65535) gy = 65535;
   const int64_t kb_per = (nkb + gy - 1) / gy;
@@ -527,9 +517,11 @@ int launch_unpack_e2m1(const uint64_t *geno, int64_t n_f, int64_t n_v, int64_t l
     return launch_unpack_blocked(geno, n_f, n_v, ld, op, kpad, snps_pad, blocked_rows, true, w,
                                  gamma, s);
   // Fused with the factors while one 128-thread block per SNP still gives the
-  // GPU enough loads in flight (152 SMs x 8 blocks); a few long rows take the
-  // flat unpack (a thread per word) and the multi-warp count kernel instead.
-  if (w != nullptr && snps_pad >= 152 * 8) {
+  // GPU enough loads in flight (152 SMs x 8 blocks), or a row is at most two
+  // words per thread, where a second launch is what would cost (256 x 1,024: 22.8
+  // -> 19.3 us per call); a few long rows take the flat unpack (a thread per
+  // word) and the multi-warp count kernel instead.
+  if (w != nullptr && (snps_pad >= 152 * 8 || kpad <= 2 * 128 * 32)) {
     if (snps_pad < n_v) return CCC_EINVAL;
     k_unpack_e2m1_w<<<static_cast<unsigned>(snps_pad), 128, 0, s>>>(geno, n_f, n_v, ld, op, kpad,
                                                                      w, gamma, counts);
