@@ -687,7 +687,8 @@ static int slabs_3way(Run3 &R) {
       const int64_t mrow0 = L.rows_pad + h * L.mask_rows;
       if (P != nullptr && b >= 2 && cudaStreamWaitEvent(ps, P->consumed[h], 0) != cudaSuccess)
         return CCC_ECUDA;
-      CCC_TRY(launch_compact3(p->geno, p->n_f, p->n_v, p->ld, cb, ms, j0, j1, ps, R.fp4));
+      CCC_TRY(launch_compact3(p->geno, p->n_f, p->n_v, p->ld, cb, ms, j0, j1,
+                              at<uint32_t>(o, L.dscratch), h, L.cbuf_slabs, R.dev.sms, ps, R.fp4));
       CCC_TRY(launch_mask3c(p->geno, p->n_f, p->n_v, p->ld, op, L.kpad, mrow0, ms, j0, j1, ps,
                             R.fp4));
       if (P != nullptr && (cudaEventRecord(P->prepared[h], ps) != cudaSuccess ||

@@ -222,8 +222,12 @@ int64_t tc3_class_cbuf_rows(int64_t n_slabs, int64_t n_v);
 int64_t tc3_class_mask_rows(int64_t j0, int64_t j1, int64_t n_v);
 // fp4: e2m1 nibbles; compacted rows of tc3_class_cap() / 2 bytes, masked rows
 // (and R) of kpad / 2 bytes.
+//                    dscratch: see launch_tally3_class; also the lists of
+//                    missing individuals of up to max_slabs slabs per batch
+//                    buffer (half 0 or 1), behind the slots.
 int launch_compact3(const uint64_t *geno, int64_t n_f, int64_t n_v, int64_t ld, uint8_t *cbuf,
-                    int32_t *missing, int64_t j0, int64_t j1, cudaStream_t s, bool fp4 = false);
+                    int32_t *missing, int64_t j0, int64_t j1, uint32_t *dscratch, int half,
+                    int64_t max_slabs, int num_sms, cudaStream_t s, bool fp4 = false);
 int launch_mask3c(const uint64_t *geno, int64_t n_f, int64_t n_v, int64_t ld, uint8_t *op,
                   int64_t kpad, int64_t mrow0, const int32_t *missing, int64_t j0, int64_t j1,
                   cudaStream_t s, bool fp4 = false);

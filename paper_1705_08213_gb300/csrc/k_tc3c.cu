@@ -16,8 +16,9 @@
 // r_ik come from one 2-way tally pass.
 //
 // Passes per batch of slabs:
-//   k_compact3  the individuals with v_j missing; when there are at most kCap
-//               of them, the count rows of every SNP restricted to them;
+//   k_missing3, k_gather3 (n_f <= 16,383), k_compact3  the individuals with v_j
+//               missing; when there are at most kCap of them, the count rows of
+//               every SNP restricted to them;
 //   k_mask3c    for the side of the slab with fewer SNPs (i < j or k > j),
 //               rows R(s, x) * s_j in e4m3 (values 0, +-1, +-2), and, when v_j
 //               has more than kCap missing entries, rows R(s, x) * [v_j missing];
@@ -1130,6 +1131,12 @@ __global__ void __launch_bounds__(wide::kThreads, 1) __cluster_dims__(2, 1, 1)
     char *const wring = rings + kEpiWarps * wide::kRingBytes + slice * wide::kWringBytes;
     const int c_first = half * (wide::kHalfK / 8);  // the warp's 8-k chunks
     const int chunks = half == 0 ? wide::kHalfK / 8 : kChunks - wide::kHalfK / 8;
+    // The warp's chunks that hold a triple (a tile at the slab's edge has rows i >= j
+    // and columns past n_v): of a small panel's tiles most are edges.
+    auto live = [&](const Sched &t) {
+      const int hi = min(8 * chunks, static_cast<int>(n_v) - t.k0() - wide::kHalfK * half);
+      return t.i0() + 64 * static_cast<int>(rank) + 16 * quarter < t.j && hi > 0 ? (hi + 7) / 8 : 0;
+    };
     int dcount = 0;
     Sched sc, pv;
     bool pv_has_d = false;
@@ -1163,8 +1170,9 @@ __global__ void __launch_bounds__(wide::kThreads, 1) __cluster_dims__(2, 1, 1)
         if (!__all_sync(0xffffffffu, got)) return false;
         tc_fence_after();
         uint32_t *to = dsc + (u & 1) * kDWords;
+        const int c_end = c_first + live(sc);
 #pragma unroll 2
-        for (int c = c_first; c < c_first + chunks; ++c) {
+        for (int c = c_first; c < c_end; ++c) {
           uint32_t v[16];
           tmem_ld_32x32b_x16(lane_base + (u & 1) * kN + 16 * c, v);
           tmem_ld_wait();
@@ -1189,9 +1197,18 @@ __global__ void __launch_bounds__(wide::kThreads, 1) __cluster_dims__(2, 1, 1)
         const bool got = mbar_wait_bounded(tfull_bar(acc), (v >> 1) & 1, status, abort_flag);
         if (!__all_sync(0xffffffffu, got)) break;
         tc_fence_after();
+        const int n = live(pv);
+        auto release = [&]() {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(tempty_bar(acc));  // the follower's is forwarded
+        };
         const uint32_t t_x = lane_base + acc * kN + 16 * c_first;
         uint32_t x[16];
-        tmem_ld_32x32b_x16(t_x, x);
+        if (n > 0)
+          tmem_ld_32x32b_x16(t_x, x);
+        else
+          release();
         ep.products();
         // Chunk c (h = its parity): its columns into the ring, the next chunk's loads, its lines.
         auto chunk = [&](int c, int h) {
@@ -1201,26 +1218,24 @@ __global__ void __launch_bounds__(wide::kThreads, 1) __cluster_dims__(2, 1, 1)
           if (MODE == 1 && (lane >> 3) == (c & 3))
             *reinterpret_cast<float2 *>(wring + 64 * h + 8 * (lane & 7)) = c < 4 ? wk[0] : wk[1];
           __syncwarp();
-          if (c + 1 < chunks) {
+          if (c + 1 < n) {
             tmem_ld_32x32b_x16(t_x + 16 * (c + 1), x);
-          } else {  // every column is in the ring
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(tempty_bar(acc));  // the follower's is forwarded
+          } else {
+            release();  // every column is in the ring
           }
           ep.fetch(f[h ^ 1], args, 8 * (c + 1), pv_has_d, slot, keep_pol);
           ep.line(args, 8 * c, 128 * h, f[h], ring, wring);
         };
 #pragma unroll 1
-        for (int c = 0; c < chunks; c += 2) {
+        for (int c = 0; c < n; c += 2) {
           chunk(c, 0);
-          if (c + 1 < chunks) chunk(c + 1, 1);
+          if (c + 1 < n) chunk(c + 1, 1);
         }
         // The rows' last, partial lines.
-        if (chunks & 1)
-          ep.line(args, 8 * chunks, 128, f[1], ring, wring);
-        else
-          ep.line(args, 8 * chunks, 0, f[0], ring, wring);
+        if (n & 1)
+          ep.line(args, 8 * n, 128, f[1], ring, wring);
+        else if (n > 0)
+          ep.line(args, 8 * n, 0, f[0], ring, wring);
       }
       if (!sc.valid) break;
       pv = sc;
@@ -1248,8 +1263,6 @@ __global__ void __launch_bounds__(wide::kThreads, 1) __cluster_dims__(2, 1, 1)
 // and in its tail.
 constexpr int kPrepThreads = 128;
 
-// FP4: the compacted rows in e2m1 nibbles, 256 individuals in 128 bytes per row.
-template <bool FP4>
 __global__ void __launch_bounds__(kPrepThreads, 9) k_compact3(const uint64_t *__restrict__ geno, int64_t n_f,
                                                   int64_t n_v, int64_t ld, int64_t j0,
                                                   uint8_t *__restrict__ cbuf,
@@ -1305,38 +1318,168 @@ __global__ void __launch_bounds__(kPrepThreads, 9) k_compact3(const uint64_t *__
     const int q = pos[idx];
     return static_cast<uint32_t>(__ldg(geno + s * ld + (q >> 5)) >> (2 * (q & 31))) & 3u;
   };
-  if constexpr (FP4) {
-    // e2m1 nibbles: 0 -> 0x0, 1 -> 0x2, 2 -> 0x4; column idx in the low nibble of
-    // byte idx / 2 for even idx.  One K stage of 256 individuals = 128 bytes.
-    constexpr int kRow = kCap / 2;
-    const int nbytes = (running + 255) / 256 * 128;
-    for (int64_t s = s_lo + warp; s < s_hi; s += kWarps) {
-      uint8_t *row0 = cbuf + (static_cast<int64_t>(blockIdx.x) * 2 * n_v + 2 * s) * kRow;
-      for (int b = lane; b < nbytes; b += 32) {
-        uint32_t n0 = 0u, n1 = 0u;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const uint32_t code = code_at(s, 2 * b + h);
-          const uint32_t r0 = code == 0u ? 4u : (code == 1u ? 2u : 0u);
-          const uint32_t r1 = code == 3u ? 4u : (code == 1u ? 2u : 0u);
-          n0 |= r0 << (4 * h);
-          n1 |= r1 << (4 * h);
-        }
-        row0[b] = static_cast<uint8_t>(n0);
-        row0[kRow + b] = static_cast<uint8_t>(n1);
-      }
+  const int ncols = (running + kBK - 1) / kBK * kBK;
+  for (int64_t s = s_lo + warp; s < s_hi; s += kWarps) {
+    uint8_t *row0 = cbuf + (static_cast<int64_t>(blockIdx.x) * 2 * n_v + 2 * s) * kCap;
+    for (int idx = lane; idx < ncols; idx += 32) {
+      const uint32_t code = code_at(s, idx);
+      // e4m3: 0 -> 0x00, 1 -> 0x38, 2 -> 0x40
+      const uint8_t e0 = code == 0u ? 0x40 : (code == 1u ? 0x38 : 0x00);
+      const uint8_t e1 = code == 3u ? 0x40 : (code == 1u ? 0x38 : 0x00);
+      row0[idx] = e0;
+      row0[kCap + idx] = e1;
     }
-  } else {
-    const int ncols = (running + kBK - 1) / kBK * kBK;
-    for (int64_t s = s_lo + warp; s < s_hi; s += kWarps) {
-      uint8_t *row0 = cbuf + (static_cast<int64_t>(blockIdx.x) * 2 * n_v + 2 * s) * kCap;
-      for (int idx = lane; idx < ncols; idx += 32) {
-        const uint32_t code = code_at(s, idx);
-        // e4m3: 0 -> 0x00, 1 -> 0x38, 2 -> 0x40
-        const uint8_t e0 = code == 0u ? 0x40 : (code == 1u ? 0x38 : 0x00);
-        const uint8_t e1 = code == 3u ? 0x40 : (code == 1u ? 0x38 : 0x00);
-        row0[idx] = e0;
-        row0[kCap + idx] = e1;
+  }
+}
+
+// The same for n_f <= kWideMaxNf in two steps that read each SNP's codes once per
+// group of slabs instead of once per slab: a compacted row takes one code from
+// each of 82 sectors of a 2 KB row (1,536 x 8,192, 1% missing), which bounded
+// k_compact3 by L2 (653 us per call; the two now 330).
+//   k_missing3  per slab of the batch: lists[slab * kCap + t] = 2 q of the t-th
+//               individual q with v_j missing, the rest kSentinel, and the count.
+//   k_gather3   a CTA holds the packed rows of its SNPs in shared memory (each
+//               followed by a word of missing codes, to which the sentinel
+//               points) and walks the slabs of its group; a half-warp takes one
+//               SNP, a lane eight of its 128 columns at a time.
+__device__ __forceinline__ uint32_t sentinel(int64_t n_f) {
+  return static_cast<uint32_t>((n_f + 15) / 16) * 32u;  // 2 q of the word after the row
+}
+
+__global__ void __launch_bounds__(kPrepThreads) k_missing3(const uint64_t *__restrict__ geno,
+                                                           int64_t n_f, int64_t ld, int64_t j0,
+                                                           uint16_t *__restrict__ lists,
+                                                           int32_t *__restrict__ missing) {
+  constexpr int kWarps = kPrepThreads / 32;
+  __shared__ int warp_tot[2][kWarps];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t j = j0 + blockIdx.x;
+  const int nw = static_cast<int>((n_f + 31) / 32);
+  uint16_t *const list = lists + static_cast<int64_t>(blockIdx.x) * kCap;
+  int running = 0;
+  for (int base = 0, it = 0; base < nw; base += kPrepThreads, it ^= 1) {
+    const int wi = base + tid;
+    uint64_t miss = 0;
+    if (wi < nw) {
+      const uint64_t v = __ldg(geno + j * ld + wi);
+      uint64_t valid = kEven;
+      const int64_t tail = n_f - static_cast<int64_t>(wi) * 32;
+      if (tail < 32) valid &= (1ull << (2 * tail)) - 1ull;
+      miss = (v >> 1) & ~v & valid;
+    }
+    const int c = __popcll(miss);
+    int x = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) warp_tot[it][warp] = x;
+    __syncthreads();
+    int before = 0, tot = 0;
+#pragma unroll
+    for (int q = 0; q < kWarps; ++q) {
+      before += q < warp ? warp_tot[it][q] : 0;
+      tot += warp_tot[it][q];
+    }
+    int o = running + before + x - c;
+    while (miss != 0 && o < kCap) {
+      const int b = __ffsll(static_cast<long long>(miss)) - 1;  // an even bit: 2 q within the word
+      list[o++] = static_cast<uint16_t>(wi * 64 + b);
+      miss &= miss - 1;
+    }
+    running += tot;
+  }
+  for (int o = running + tid; o < kCap; o += kPrepThreads) list[o] = static_cast<uint16_t>(sentinel(n_f));
+  if (tid == 0) missing[blockIdx.x] = running;
+}
+
+constexpr int kGatherThreads = 256;
+constexpr int kGatherSnps = 64;             // SNPs per CTA at most
+constexpr size_t kGatherBytes = 100 * 1024;  // of shared memory for their rows
+
+// 32-bit words of a SNP's row in shared memory: the codes, the missing word, odd.
+__host__ __device__ inline int gather_stride(int64_t n_f) {
+  return static_cast<int>((n_f + 15) / 16 + 1) | 1;
+}
+inline int gather_snps(int64_t n_f) {
+  const int n = static_cast<int>(kGatherBytes / (4 * static_cast<size_t>(gather_stride(n_f)))) / 16 * 16;
+  return n < 16 ? 16 : n > kGatherSnps ? kGatherSnps : n;
+}
+
+template <bool FP4>
+__global__ void __launch_bounds__(kGatherThreads, 2)
+    k_gather3(const uint64_t *__restrict__ geno, int64_t n_f, int64_t n_v, int64_t ld,
+              const uint16_t *__restrict__ lists, const int32_t *__restrict__ missing, int slabs,
+              uint8_t *__restrict__ cbuf, int snps) {
+  extern __shared__ uint32_t rows[];
+  __shared__ __align__(16) uint16_t slist[2][kCap];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int stride = gather_stride(n_f);
+  const int words = static_cast<int>((n_f + 15) / 16);
+  const int64_t s0 = static_cast<int64_t>(blockIdx.x) * snps;
+  const int mine = n_v - s0 < snps ? static_cast<int>(n_v - s0) : snps;
+  const uint32_t *g32 = reinterpret_cast<const uint32_t *>(geno);
+  constexpr int kW = kGatherThreads / 32;
+  for (int s = warp; s < mine; s += 4 * kW)  // four rows' loads in flight
+    for (int k = lane; k < stride; k += 32) {
+      uint32_t v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        v[u] = k < words && s + u * kW < mine ? __ldg(g32 + (s0 + s + u * kW) * ld * 2 + k) : 0xAAAAAAAAu;
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (s + u * kW < mine) rows[(s + u * kW) * stride + k] = v[u];
+    }
+  constexpr int kRow = FP4 ? kCap / 2 : kCap;
+  const int l16 = lane & 15;
+  // Slabs blockIdx.y, + gridDim.y, ...: the next slab's list is fetched during this one's rows.
+  auto fetch = [&](int x, int buf) {
+    if (x < slabs && tid < kCap / 8)
+      reinterpret_cast<uint4 *>(slist[buf])[tid] =
+          __ldg(reinterpret_cast<const uint4 *>(lists + static_cast<int64_t>(x) * kCap) + tid);
+  };
+  fetch(blockIdx.y, 0);
+  int buf = 0;
+  for (int x = blockIdx.y; x < slabs; x += gridDim.y, buf ^= 1) {
+    const int c = __ldg(missing + x);
+    __syncthreads();  // the list (and, the first time, the rows) are there; the other is free
+    fetch(x + gridDim.y, buf ^ 1);
+    if (c == 0 || c > kCap) continue;
+    uint8_t *const out = cbuf + (static_cast<int64_t>(x) * 2 * n_v + 2 * s0) * kRow;
+    // Columns from 128 on only when the tiles read them (whole 128-byte K stages).
+    const int blocks = FP4 || c > 128 ? 2 : 1;
+    for (int s = 2 * warp + (lane >> 4); s < mine; s += kGatherThreads / 16) {
+      const uint32_t *row = rows + s * stride;
+      uint8_t *const d0 = out + static_cast<int64_t>(2 * s) * kRow;
+      for (int b = 0; b < blocks; ++b) {
+        uint32_t codes = 0xAAAAu;
+        if (128 * b < c) {
+          const uint4 q = *reinterpret_cast<const uint4 *>(slist[buf] + 128 * b + 8 * l16);
+          const uint32_t e[4] = {q.x, q.y, q.z, q.w};
+          codes = 0u;
+#pragma unroll
+          for (int t = 0; t < 8; ++t) {
+            const uint32_t p = t & 1 ? e[t >> 1] >> 16 : e[t >> 1] & 0xFFFFu;
+            codes |= ((row[p >> 5] >> (p & 31)) & 3u) << (2 * t);
+          }
+        }
+        // Codes to nibbles: the FP4 counts, or selectors of the e4m3 bytes.
+        uint32_t y = (codes | (codes << 8)) & 0x00FF00FFu;
+        y = (y | (y << 4)) & 0x0F0F0F0Fu;
+        y = (y | (y << 2)) & 0x33333333u;
+        if constexpr (FP4) {
+          const uint32_t h = y >> 1;
+          const uint32_t het = (y & ~h & 0x11111111u) << 1;
+          reinterpret_cast<uint32_t *>(d0)[16 * b + l16] = het | ((~(y | h) & 0x11111111u) << 2);
+          reinterpret_cast<uint32_t *>(d0 + kRow)[16 * b + l16] = het | ((y & h & 0x11111111u) << 2);
+        } else {
+          // e4m3 bytes of rho(0), rho(1) by code: 0x40 = 2, 0x38 = 1.
+          reinterpret_cast<uint2 *>(d0)[16 * b + l16] =
+              make_uint2(__byte_perm(0x00003840u, 0u, y), __byte_perm(0x00003840u, 0u, y >> 16));
+          reinterpret_cast<uint2 *>(d0 + kRow)[16 * b + l16] =
+              make_uint2(__byte_perm(0x40003800u, 0u, y), __byte_perm(0x40003800u, 0u, y >> 16));
+        }
       }
     }
   }
@@ -1385,66 +1528,57 @@ __device__ __forceinline__ void class_masks_e2m1(uint64_t w, bool missing_mode, 
 //   mrow(j) + 2 side + 2 t + x    = R(s, x) * [v_j missing]  (only when v_j has
 //                                                          more than kCap missing)
 // in the operand buffer op (rows of kpad bytes; R occupies the first rows).
-// A CTA takes every gridDim.x-th row of its slab; a thread 16 bytes at a time.
+// A CTA's threads form groups of tpr that take four consecutive rows at a time
+// (four loads per thread in flight), a thread 16 bytes of each; the masks of its
+// individuals are formed once for all its rows.  Bound by its writes: 4.8 GB at
+// 1,536 x 8,192 in 0.79 ms (6.1 TB/s; 1.17 ms with a CTA per few rows).
 // FP4: e2m1 rows of kpad / 2 bytes, 16 bytes = the 32 individuals of one packed
 // word; the sign of a nibble is its bit 3.
+constexpr int kMaskThreads = 256;
 template <bool FP4>
-__global__ void __launch_bounds__(kPrepThreads, 9) k_mask3c(const uint64_t *__restrict__ geno, int64_t n_f,
-                                                int64_t n_v, int64_t ld, uint8_t *__restrict__ op,
-                                                int64_t kpad, int64_t mrow0, int64_t j0,
-                                                const int32_t *__restrict__ missing) {
+__global__ void __launch_bounds__(kMaskThreads) k_mask3c(const uint64_t *__restrict__ geno,
+                                                         int64_t n_f, int64_t n_v, int64_t ld,
+                                                         uint8_t *__restrict__ op, int64_t kpad,
+                                                         int64_t mrow0, int64_t j0,
+                                                         const int32_t *__restrict__ missing,
+                                                         int tpr) {
   const int64_t j = j0 + blockIdx.y;
-  const int64_t side = j < n_v - 1 - j ? j : n_v - 1 - j;
+  const int side2 = 2 * static_cast<int>(j < n_v - 1 - j ? j : n_v - 1 - j);
   const bool im = 2 * j <= n_v - 1;
-  const bool dfull = __ldg(missing + blockIdx.y) > kCap;
-  const int64_t rows = (dfull ? 4 : 2) * side;
-  const int64_t row_bytes = FP4 ? kpad / 2 : kpad;
-  const int chunks = static_cast<int>(row_bytes / 16);
-  const int64_t mrow = mrow0 + 4 * (mask_prefix(j, n_v) - mask_prefix(j0, n_v));
-  const int64_t words = (n_f + 31) / 32;
+  const int parts = __ldg(missing + blockIdx.y) > kCap ? 2 : 1;
+  const int chunks = static_cast<int>((FP4 ? kpad / 2 : kpad) / 16);
+  const int words = static_cast<int>((n_f + 31) / 32);
   const uint64_t *__restrict__ gj = geno + j * ld;
-  // Rows r, r + gridDim.x, ... in groups of 4 so that 8 loads per thread are in flight.
+  const uint4 *const src = reinterpret_cast<const uint4 *>(op) + (im ? 0 : 2 * (j + 1)) * chunks;
+  uint4 *const dst = reinterpret_cast<uint4 *>(op) +
+                     (mrow0 + 4 * (mask_prefix(j, n_v) - mask_prefix(j0, n_v))) * chunks;
   constexpr int kRows = 4;
-  for (int64_t r0 = blockIdx.x; r0 < rows; r0 += static_cast<int64_t>(gridDim.x) * kRows) {
-    const uint4 *src[kRows];
-    uint4 *dst[kRows];
-    bool dm[kRows], live[kRows];
-#pragma unroll
-    for (int u = 0; u < kRows; ++u) {
-      const int64_t ru = r0 + static_cast<int64_t>(u) * gridDim.x;
-      live[u] = ru < rows;
-      const int64_t r = live[u] ? ru : r0;
-      dm[u] = r >= 2 * side;
-      const int64_t rt = dm[u] ? r - 2 * side : r;
-      const int64_t sn = im ? (rt >> 1) : j + 1 + (rt >> 1);
-      src[u] = reinterpret_cast<const uint4 *>(op + (2 * sn + (rt & 1)) * row_bytes);
-      dst[u] = reinterpret_cast<uint4 *>(op + (mrow + r) * row_bytes);
-    }
-    for (int c = threadIdx.x; c < chunks; c += blockDim.x) {
-      uint32_t ks[4], ns[4], km[4], nm[4];
+  const int group = threadIdx.x / tpr, lane = threadIdx.x - group * tpr;
+  const int step = static_cast<int>(gridDim.x) * (kMaskThreads / tpr) * kRows;
+  for (int part = 0; part < parts; ++part) {  // rows * s_j, then rows * [v_j missing]
+    uint4 *const to = dst + static_cast<int64_t>(part) * side2 * chunks;
+    for (int c = lane; c < chunks; c += tpr) {
+      uint32_t keep[4], neg[4];
       if (FP4) {
-        const uint64_t w = c < words ? __ldg(gj + c) : 0ull;
-        class_masks_e2m1(w, false, ks, ns);
-        class_masks_e2m1(w, true, km, nm);
+        class_masks_e2m1(c < words ? __ldg(gj + c) : 0ull, part == 1, keep, neg);
       } else {
         const int wi = c >> 1;
-        uint32_t w = 0u;
-        if (wi < words) w = static_cast<uint32_t>(__ldg(gj + wi) >> (32 * (c & 1)));
-        class_masks(w, false, ks, ns);
-        class_masks(w, true, km, nm);
+        const uint32_t w = wi < words ? static_cast<uint32_t>(__ldg(gj + wi) >> (32 * (c & 1))) : 0u;
+        class_masks(w, part == 1, keep, neg);
       }
-      uint4 v[kRows];
+      for (int r = (static_cast<int>(blockIdx.x) * (kMaskThreads / tpr) + group) * kRows; r < side2;
+           r += step) {
+        uint4 v[kRows];
 #pragma unroll
-      for (int u = 0; u < kRows; ++u) v[u] = live[u] ? __ldg(src[u] + c) : make_uint4(0u, 0u, 0u, 0u);
+        for (int u = 0; u < kRows; ++u)
+          v[u] = r + u < side2 ? __ldg(src + static_cast<int64_t>(r + u) * chunks + c)
+                               : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-      for (int u = 0; u < kRows; ++u) {
-        if (!live[u]) continue;
-        uint4 o;
-        o.x = (v[u].x & (dm[u] ? km[0] : ks[0])) | (dm[u] ? nm[0] : ns[0]);
-        o.y = (v[u].y & (dm[u] ? km[1] : ks[1])) | (dm[u] ? nm[1] : ns[1]);
-        o.z = (v[u].z & (dm[u] ? km[2] : ks[2])) | (dm[u] ? nm[2] : ns[2]);
-        o.w = (v[u].w & (dm[u] ? km[3] : ks[3])) | (dm[u] ? nm[3] : ns[3]);
-        dst[u][c] = o;
+        for (int u = 0; u < kRows; ++u)
+          if (r + u < side2)
+            to[static_cast<int64_t>(r + u) * chunks + c] =
+                make_uint4((v[u].x & keep[0]) | neg[0], (v[u].y & keep[1]) | neg[1],
+                           (v[u].z & keep[2]) | neg[2], (v[u].w & keep[3]) | neg[3]);
       }
     }
   }
@@ -1452,6 +1586,7 @@ __global__ void __launch_bounds__(kPrepThreads, 9) k_mask3c(const uint64_t *__re
 
 }  // namespace
 
+bool tc3_class_table16(int64_t n_f) { return n_f <= kWideMaxNf; }
 int64_t tc3_class_cbuf_rows(int64_t n_slabs, int64_t n_v) { return n_slabs * 2 * n_v; }
 int64_t tc3_class_cap() { return kCap; }
 int64_t tc3_class_mask_rows(int64_t j0, int64_t j1, int64_t n_v) {
@@ -1459,16 +1594,49 @@ int64_t tc3_class_mask_rows(int64_t j0, int64_t j1, int64_t n_v) {
 }
 
 int launch_compact3(const uint64_t *geno, int64_t n_f, int64_t n_v, int64_t ld, uint8_t *cbuf,
-                    int32_t *missing, int64_t j0, int64_t j1, cudaStream_t s, bool fp4) {
+                    int32_t *missing, int64_t j0, int64_t j1, uint32_t *dscratch, int half,
+                    int64_t max_slabs, int num_sms, cudaStream_t s, bool fp4) {
   if (j1 <= j0) return CCC_OK;
+  // The lists go behind the D slots of the CTAs that this GPU can run.
+  const int64_t room = (wide::kMaxCtas - static_cast<int64_t>(num_sms)) * 2 * wide::kDWords * 4;
+  if (tc3_class_table16(n_f) && 2 * max_slabs * kCap * 2 <= room) {
+    uint16_t *const lists =
+        reinterpret_cast<uint16_t *>(dscratch + static_cast<int64_t>(num_sms) * 2 * wide::kDWords) +
+        static_cast<int64_t>(half) * max_slabs * kCap;
+    const int slabs = static_cast<int>(j1 - j0);
+    k_missing3<<<static_cast<unsigned>(slabs), kPrepThreads, 0, s>>>(geno, n_f, ld, j0, lists,
+                                                                     missing);
+    const int rc = note_launch();
+    if (rc != CCC_OK) return rc;
+    static bool attr_set[kMaxDevices] = {};
+    const int dev = current_device();
+    if (dev < 0) return CCC_ECUDA;
+    if (!attr_set[dev]) {
+      if (cudaFuncSetAttribute(k_gather3<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               static_cast<int>(kGatherBytes)) != cudaSuccess ||
+          cudaFuncSetAttribute(k_gather3<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               static_cast<int>(kGatherBytes)) != cudaSuccess)
+        return CCC_ECUDA;
+      attr_set[dev] = true;
+    }
+    const int snps = gather_snps(n_f);
+    const int64_t gx = cdiv(n_v, snps);
+    int64_t gy = cdiv(4 * static_cast<int64_t>(num_sms), gx);  // two resident CTAs per SM, twice
+    if (gy > slabs) gy = slabs;
+    const dim3 grid(static_cast<unsigned>(gx), static_cast<unsigned>(gy), 1);
+    const size_t smem = 4 * static_cast<size_t>(gather_stride(n_f)) * static_cast<size_t>(snps);
+    if (fp4)
+      k_gather3<true><<<grid, kGatherThreads, smem, s>>>(geno, n_f, n_v, ld, lists, missing, slabs,
+                                                         cbuf, snps);
+    else
+      k_gather3<false><<<grid, kGatherThreads, smem, s>>>(geno, n_f, n_v, ld, lists, missing, slabs,
+                                                          cbuf, snps);
+    return note_launch();
+  }
+  if (fp4) return CCC_EUNSUPPORTED;
   const int snps_per_cta = 64;
   const dim3 grid(static_cast<unsigned>(j1 - j0), static_cast<unsigned>(cdiv(n_v, snps_per_cta)), 1);
-  if (fp4)
-    k_compact3<true><<<grid, kPrepThreads, 0, s>>>(geno, n_f, n_v, ld, j0, cbuf, missing,
-                                                   snps_per_cta);
-  else
-    k_compact3<false><<<grid, kPrepThreads, 0, s>>>(geno, n_f, n_v, ld, j0, cbuf, missing,
-                                                    snps_per_cta);
+  k_compact3<<<grid, kPrepThreads, 0, s>>>(geno, n_f, n_v, ld, j0, cbuf, missing, snps_per_cta);
   return note_launch();
 }
 
@@ -1476,16 +1644,20 @@ int launch_mask3c(const uint64_t *geno, int64_t n_f, int64_t n_v, int64_t ld, ui
                   int64_t kpad, int64_t mrow0, const int32_t *missing, int64_t j0, int64_t j1,
                   cudaStream_t s, bool fp4) {
   if (j1 <= j0) return CCC_OK;
-  // About 8 CTAs per SM in total; each slab's rows are spread over bx CTAs.
-  int64_t bx = cdiv(8 * 160, j1 - j0);
-  if (bx < 2) bx = 2;
-  if (bx > 256) bx = 256;
-  const dim3 grid(static_cast<unsigned>(bx), static_cast<unsigned>(j1 - j0), 1);
   if (fp4 && kpad % 256 != 0) return CCC_EINVAL;
+  const int64_t chunks = (fp4 ? kpad / 2 : kpad) / 16;
+  int tpr = 32;  // threads per row: whole warps, a power of two
+  while (tpr < kMaskThreads && tpr < chunks) tpr *= 2;
+  // About 16 CTAs per SM in total, each slab's rows spread over bx of them.
+  const int64_t most = cdiv(n_v, (kMaskThreads / tpr) * 4);  // 2 x side <= n_v rows, 4 per group
+  int64_t bx = cdiv(16 * 152, j1 - j0);
+  if (bx < 2) bx = 2;
+  if (bx > most) bx = most;
+  const dim3 grid(static_cast<unsigned>(bx), static_cast<unsigned>(j1 - j0), 1);
   if (fp4)
-    k_mask3c<true><<<grid, kPrepThreads, 0, s>>>(geno, n_f, n_v, ld, op, kpad, mrow0, j0, missing);
+    k_mask3c<true><<<grid, kMaskThreads, 0, s>>>(geno, n_f, n_v, ld, op, kpad, mrow0, j0, missing, tpr);
   else
-    k_mask3c<false><<<grid, kPrepThreads, 0, s>>>(geno, n_f, n_v, ld, op, kpad, mrow0, j0, missing);
+    k_mask3c<false><<<grid, kMaskThreads, 0, s>>>(geno, n_f, n_v, ld, op, kpad, mrow0, j0, missing, tpr);
   return note_launch();
 }
 
@@ -1559,8 +1731,6 @@ static int launch_tally3_class_w(const Tally3Args &a, const uint8_t *op, int64_t
     return launch_wide_mode<1, FP4>(tmOp, tmC, ca, sp, tiles, num_sms, s);
   return launch_wide_mode<2, FP4>(tmOp, tmC, ca, sp, tiles, num_sms, s);
 }
-
-bool tc3_class_table16(int64_t n_f) { return n_f <= kWideMaxNf; }
 
 int64_t tc3_class_dscratch_bytes() {
   return static_cast<int64_t>(wide::kMaxCtas) * 2 * wide::kDWords * 4;

@@ -58,3 +58,32 @@ def test_arrays_at_any_16_bytes(n_v, n_f, missing, off_t, off_c, norm, operand):
         only = torch.full((cnt, 8), -7, dtype=torch.int32, device="cuda")
         ccc.ccc3_tally(g, n_f, j0, j1, only, opts)
         assert torch.equal(only, t)
+
+
+@pytest.mark.parametrize("operand", [1, 2])
+@pytest.mark.parametrize("n_v,n_f", [(19, 600), (37, 2050), (18, 16383)])
+def test_missing_counts_at_the_edges_of_the_lists(n_v, n_f, operand):
+    """Middle SNPs with exactly 0, 1, 127 .. 129, 255 .. 257 and more missing entries: the compacted
+    rows' two halves, their capacity, and the masked rows that take over beyond it."""
+    import numpy as np
+    import torch
+
+    import paper_1705_08213_gb300 as ccc
+    geno = synth.panel_hwe(n_v, n_f, seed=5 * n_v, p_missing=0.0, pad_seed=2)
+    rng = np.random.default_rng(n_v)
+    for j in range(n_v):
+        for q in rng.choice(n_f, (0, 1, 127, 128, 129, 255, 256, 257, n_f // 2)[j % 9], replace=False):
+            w, b = divmod(int(q), 32)
+            geno[j, w] = (geno[j, w] & ~(np.uint64(3) << np.uint64(2 * b))) | (np.uint64(2) << np.uint64(2 * b))
+    g = to_device(geno)
+    opts = ccc.ccc_opts_default(operand=operand)
+    ws = workspace(ccc.ccc_workspace_size(g, n_f, opts, ccc.CCC_OP_3WAY))
+    opts = ccc.ccc_opts_default(operand=operand, workspace=ws)
+    count = ccc.ccc3_count(n_v, 0, n_v)
+    t = torch.full((count, 8), -7, dtype=torch.int32, device="cuda")
+    c = torch.full((count, 8), -7.0, dtype=torch.float32, device="cuda")
+    ccc.ccc3_tally_metric(g, n_f, 0, n_v, t, c, opts)
+    assert ccc.ccc_status(opts) == ccc.CCC_OK
+    et, ec = oracle.ccc3_slabs(geno, n_f)
+    assert_tally_equal(t.cpu().numpy(), et)
+    assert_ccc_close(c.cpu().numpy(), ec)
