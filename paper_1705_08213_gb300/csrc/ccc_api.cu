@@ -1067,10 +1067,10 @@ static int run_multi(const ccc_panel_multi *p, int32_t *tally, float *out_ccc, c
   const MultiLayout L = fp4 ? make_multi_layout(p->n_f, p->n_v, ns, true, true) : L8;
   if (p->n_v < 2) return CCC_OK;
   float *w = at<float>(o, L.w);
-  if (out_ccc != nullptr && o->norm == CCC_NORM_PERSNP)
-    CCC_TRY(launch_multi_counts(p->geno, p->n_f, p->n_v, p->ld, ns, nullptr, w, o->gamma, s));
+  const bool want_w = out_ccc != nullptr && o->norm == CCC_NORM_PERSNP;
   uint8_t *op = at<uint8_t>(o, L.op);
-  CCC_TRY(launch_multi_unpack(p->geno, p->n_f, p->n_v, p->ld, ns, op, L.kpad, L.rows_pad, s, fp4));
+  CCC_TRY(launch_multi_unpack(p->geno, p->n_f, p->n_v, p->ld, ns, op, L.kpad, L.rows_pad, s, fp4,
+                              want_w ? w : nullptr, o->gamma));
   if (split > 1) {
     // Partial tallies of the K parts summed into the zeroed output; CCC values
     // from the complete tallies.
@@ -1877,10 +1877,10 @@ int ccc2_multi_stream(const ccc_panel_multi *p, int n_phases, int32_t *host_tall
   const size_t slot0 = align_up(L8.total, 1024);  // as ccc2_multi_stream_workspace_size
   // Preparation once for all phases.
   float *w = at<float>(o, L.w);
-  if (want_ccc && o->norm == CCC_NORM_PERSNP)
-    CCC_TRY(launch_multi_counts(p->geno, p->n_f, p->n_v, p->ld, ns, nullptr, w, o->gamma, s));
+  const bool want_w = want_ccc && o->norm == CCC_NORM_PERSNP;
   uint8_t *op = at<uint8_t>(o, L.op);
-  CCC_TRY(launch_multi_unpack(p->geno, p->n_f, p->n_v, p->ld, ns, op, L.kpad, L.rows_pad, s, fp4));
+  CCC_TRY(launch_multi_unpack(p->geno, p->n_f, p->n_v, p->ld, ns, op, L.kpad, L.rows_pad, s, fp4,
+                              want_w ? w : nullptr, o->gamma));
   int64_t bounds[1025];
   phase_bounds(p->n_v, n_phases, bounds, multi_block_rows(ns));
   for (int ph = 0; ph < n_phases; ++ph) {

@@ -252,10 +252,11 @@ int launch_multi_counts(const uint8_t *geno, int64_t n_f, int64_t n_v, int64_t l
                         int32_t *counts, float *w, double gamma, cudaStream_t st);
 int launch_multi_factors(const int32_t *counts, int64_t n_v, int s, float *w, double gamma,
                          cudaStream_t st);
-// fp4: e2m1 rows of kpad / 2 bytes (kpad a multiple of 256).
+// fp4 (s <= 8): e2m1 rows of kpad / 2 bytes (kpad a multiple of 256).  w != null:
+// also the factors of launch_multi_counts (fp4: from the same read).
 int launch_multi_unpack(const uint8_t *geno, int64_t n_f, int64_t n_v, int64_t ld, int s,
                         uint8_t *op, int64_t kpad, int64_t rows_pad, cudaStream_t st,
-                        bool fp4 = false);
+                        bool fp4 = false, float *w = nullptr, double gamma = 0.0);
 // Tallies and, when out_ccc is set, CCC values of the pairs with
 // i_begin <= i < i_end (s*s each), pair (i, j) at pair_index(i, j) - pair0.
 // split > 1 (whole triangle only): the K stages in `split` parts whose partial
