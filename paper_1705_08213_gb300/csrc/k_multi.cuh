@@ -76,8 +76,31 @@ template <int S, int NBQ = 8>
 struct EpiMultiT {
   using Params = MultiArgs;
   static constexpr int PW = snps_per_quarter(S);
-  // The PERSNP factors w_j of the warp's NBQ / 2 quarters of markers.
-  static constexpr int STAGE_BYTES_PER_WARP = (NBQ / 2) * 32 * 4;
+  static constexpr int CHUNKS = NBQ / 2;  // of a warp
+  // FP4 tiles with S = 2 or odd S: the outputs leave through shared memory
+  // (put_chunk).  Otherwise (direct) a lane stores its own row of the table in
+  // pieces of 16 bytes (S = 4, 8) or 8 (S = 6), which make up runs of S^2 words
+  // anyway; the stage's traffic then costs more than it saves, because it
+  // competes with the MMAs' operand reads.  GB300, us per call, direct / staged:
+  //   S = 4, 10,000 x 16,384: 4536 / 4751; 3,000 x 4,000: 159 / 217
+  //   S = 8, 2,000 x 8,000: 460 / 447; 3,000 x 2,000, JOINT: 668 / 824
+  //   S = 6, 3,000 x 4,000: 487 / 461; 3,000 x 1,500, JOINT: 455 / 551
+  // The e4m3 tiles' operand stages leave no room for it.  Loading all of a warp's
+  // chunks and releasing the accumulator before the first is stored was slower
+  // for every S (S = 4, 10,000 x 16,384: 4601; S = 3, 3,000 x 4,000: 175 for 168).
+  static constexpr bool STAGED = NBQ == kMultiRectQ && (S == 2 || S % 2 == 1);
+  // A marker i's words of one chunk, RUN = PW S^2, start RUN_LD words apart:
+  // RUN_LD = S^2 (mod 32), so that the rows that the lanes (u, a) write at
+  // u RUN_LD + a S fall on different banks.
+  static constexpr int SS = S * S;
+  static constexpr int RUN = PW * SS;
+  static constexpr int RUN_LD = SS % 32 + (RUN - SS % 32 + 31) / 32 * 32;
+  static constexpr int W = S % 2 == 0 ? 4 : 1;  // words a lane stores
+  static constexpr int NV = RUN / W;
+  static constexpr int LPR = NV <= 16 ? 16 : 32;  // lanes of a run
+  static constexpr int OUT_WORDS = STAGED ? (PW * RUN_LD + 3) / 4 * 4 : 0;
+  // Behind them, the PERSNP factors w_j of the warp's NBQ / 2 quarters of markers.
+  static constexpr int STAGE_BYTES_PER_WARP = (OUT_WORDS + CHUNKS * 32) * 4;
   using Sched = std::conditional_t<NBQ == 8, TriSchedPair,
                                    RectSchedT<8 * PW, NBQ * PW, 32 * NBQ>>;
 
@@ -93,8 +116,9 @@ struct EpiMultiT {
                               float *stage, tcp::NoEarly, bool) {
     static_assert(!PRELOAD, "s-state tiles run on the two-accumulator pipeline");
     static_assert(NBQ % 2 == 0, "two column halves");
-    const int cb = (c0 / NC) * (NBQ / 2);
-    const int ce = cb + NBQ / 2;
+    const int cb = (c0 / NC) * CHUNKS;
+    const int ce = cb + CHUNKS;
+    float *const wstage = stage + OUT_WORDS;
     const int u = lane / S;
     const int a = lane - u * S;
     const int64_t n_v = args.n_v;
@@ -112,12 +136,101 @@ struct EpiMultiT {
     const int64_t jw0 = (NBQ * static_cast<int64_t>(sc.J) + cb) * PW;
     if (want_ccc && persnp) {
       __syncwarp();  // the previous tile's reads are done
-      for (int k = lane; k < (NBQ / 2) * PW * S; k += 32) {
+      for (int k = lane; k < CHUNKS * PW * S; k += 32) {
         const int64_t e = jw0 * S + k;
-        stage[k] = e < n_v * S ? __ldg(args.w + e) : 1.f;
+        wstage[k] = e < n_v * S ? __ldg(args.w + e) : 1.f;
       }
       __syncwarp();
     }
+    // Row a of the table of (i, j0 + jl) as counts; the sums that its value needs.
+    struct Sums {
+      int32_t n4, rs, col[S];
+    };
+    auto row = [&](const uint32_t *v, int (&r)[S]) {
+#pragma unroll
+      for (int b = 0; b < S; ++b) r[b] = __float2int_rn(__uint_as_float(v[b]));
+    };
+    auto sums = [&](const int (&r)[S]) {
+      Sums m;
+      m.rs = 0;
+#pragma unroll
+      for (int b = 0; b < S; ++b) m.rs += r[b];
+      // 4 n_ij = sum over the pair's table: the row sums of SNP i's s lanes.
+      m.n4 = 0;
+#pragma unroll
+      for (int k = 0; k < S; ++k) m.n4 += __shfl_sync(0xffffffffu, m.rs, src0 + k);
+      if (want_ccc && !persnp) {
+#pragma unroll
+        for (int b = 0; b < S; ++b) {
+          m.col[b] = 0;
+#pragma unroll
+          for (int k = 0; k < S; ++k) m.col[b] += __shfl_sync(0xffffffffu, r[b], src0 + k);
+        }
+      }
+      return m;
+    };
+    auto values = [&](const int (&r)[S], const Sums &m, const float *wjs, float (&cv)[S]) {
+      const float d = m.n4 == 0 ? 1.f : static_cast<float>(m.n4);
+      const float inv = rcp_count(d);
+      if (persnp) {
+#pragma unroll
+        for (int b = 0; b < S; ++b)
+          cv[b] = __fmul_rn(__fmul_rn(__fmul_rn(static_cast<float>(r[b]), inv), wi), wjs[b]);
+      } else {
+        const float wia = joint_factor(static_cast<float>(m.rs), d, inv, args.gamma);
+#pragma unroll
+        for (int b = 0; b < S; ++b) {
+          const float wjb = joint_factor(static_cast<float>(m.col[b]), d, inv, args.gamma);
+          cv[b] = __fmul_rn(__fmul_rn(div_count(static_cast<float>(r[b]), d, inv), wia), wjb);
+        }
+      }
+    };
+    // Each lane stores its own row of the chunk's tables.
+    auto direct = [&](const uint32_t *v, int c) {
+      // Column chunk c = 32 rows of the B block: its quarter c.
+      const int64_t j0 = (NBQ * static_cast<int64_t>(sc.J) + c) * PW;
+#pragma unroll
+      for (int jl = 0; jl < PW; ++jl) {
+        const int64_t j = j0 + jl;
+        int r[S];
+        row(v + jl * S, r);
+        const Sums m = sums(r);
+        if (!(row_ok && i < j && j < n_v && i >= args.i_begin && i < args.i_end)) continue;
+        if (!CCC_IN_BOUNDS(row_base + j - args.pair0, args.out_len, args.status)) continue;
+        const int64_t base = (row_base + j - args.pair0) * SS + a * S;
+        store_row<S>(args.tally + base, r);
+        if (!want_ccc) continue;
+        float cv[S];
+        values(r, m, wstage + ((c - cb) * PW + jl) * S, cv);
+        store_row<S>(args.ccc + base, cv);
+      }
+    };
+    auto staged = [&](const uint32_t *v, int c) {
+      const int64_t i0 = i - u;
+      const int64_t j0 = (NBQ * static_cast<int64_t>(sc.J) + c) * PW;
+      __syncwarp();  // the previous reads of the stage are done
+#pragma unroll
+      for (int jl = 0; jl < PW; ++jl) {
+        int r[S];
+        row(v + jl * S, r);
+        if (u < PW) put_row(reinterpret_cast<int *>(stage) + u * RUN_LD + jl * SS + a * S, r);
+      }
+      __syncwarp();
+      put_chunk(args, i0, j0, lane, reinterpret_cast<const int *>(stage), args.tally);
+      if (!want_ccc) return;
+      __syncwarp();
+#pragma unroll
+      for (int jl = 0; jl < PW; ++jl) {
+        int r[S];
+        row(v + jl * S, r);
+        const Sums m = sums(r);
+        float cv[S];
+        values(r, m, wstage + ((c - cb) * PW + jl) * S, cv);
+        if (u < PW) put_row(stage + u * RUN_LD + jl * SS + a * S, cv);
+      }
+      __syncwarp();
+      put_chunk(args, i0, j0, lane, stage, args.ccc);
+    };
     for (int c = cb; c < ce; ++c) {
       uint32_t v[32];
       tmem_ld_32x32b_x32(t_base + c * 32, v);
@@ -126,55 +239,76 @@ struct EpiMultiT {
         tc_fence_before();
         mbar_arrive_cluster(release_cluster_bar);
       }
-      // Column chunk c = 32 rows of the B block: its quarter c.
-      const int64_t j0 = (NBQ * static_cast<int64_t>(sc.J) + c) * PW;
+      if constexpr (STAGED)
+        staged(v, c);
+      else
+        direct(v, c);
+    }
+  }
+
+  // s consecutive words into the stage, as wide as their alignment allows.
+  template <typename T>
+  __device__ __forceinline__ static void put_row(T *dst, const T (&v)[S]) {
+    constexpr int R = S % 2 == 0 ? 2 : 1;
+    struct alignas(4 * R) Vec {
+      T x[R];
+    };
 #pragma unroll
-      for (int jl = 0; jl < PW; ++jl) {
-        const int64_t j = j0 + jl;
-        int32_t r[S];
-        int32_t rs = 0;
+    for (int b = 0; b < S; b += R) {
+      Vec t;
 #pragma unroll
-        for (int b = 0; b < S; ++b) {
-          r[b] = __float2int_rn(__uint_as_float(v[jl * S + b]));
-          rs += r[b];
+      for (int q = 0; q < R; ++q) t.x[q] = v[b + q];
+      *reinterpret_cast<Vec *>(dst + b) = t;
+    }
+  }
+
+  // One chunk of one array from the stage to global memory.  For each of the
+  // warp's markers i the words of the pairs (i, j0 .. j0 + PW - 1) are contiguous
+  // there, so the lanes store them side by side: 16 bytes each for S = 2 (a
+  // pair's 4 words are one 16-byte unit), words for odd S.  When each
+  // lane stored its own row of the table, an instruction wrote 32 pieces of at
+  // most 8 bytes in as many 128-byte lines as the warp has markers.
+  // GB300, 3,000 markers, us per call, direct -> staged:
+  //   4,000 individuals:  S = 2: 98 -> 85, 3: 235 -> 168, 5 (JOINT): 504 -> 426, 7: 979 -> 674
+  //   16,384 individuals: S = 2: 174 -> 171, 3: 340 -> 338, 5: 977 -> 880, 7: 1984 -> 1744
+  template <typename T>
+  __device__ __forceinline__ static void put_chunk(const MultiArgs &args, int64_t i0, int64_t j0,
+                                                   int lane, const T *stage, T *out) {
+    static_assert(PW % (32 / LPR) == 0 && (W == 1 || RUN_LD % 4 == 0), "whole runs and units");
+    struct alignas(4 * W) Vec {
+      T x[W];
+    };
+    const int64_t n_v = args.n_v;
+    const int el = (lane & (LPR - 1)) * W;
+    const int hi = n_v - j0 < PW ? static_cast<int>(n_v - j0) : PW;  // j < n_v
+#pragma unroll 2
+    for (int ul = LPR == 32 ? 0 : lane / LPR; ul < PW; ul += 32 / LPR) {
+      const int64_t i = i0 + ul;
+      const bool ok = i < n_v && i >= args.i_begin && i < args.i_end;
+      const int64_t pair = i * (2 * n_v - i - 1) / 2 - i - 1 + j0 - args.pair0;  // (i, j0)
+      // i < j: words from e0 on.
+      const int e0 = i < j0 ? 0 : i - j0 < PW ? static_cast<int>(i + 1 - j0) * SS : RUN;
+      const int e1 = ok ? hi * SS : 0;
+      T *const dst = out + pair * SS;
+      const T *const src = stage + ul * RUN_LD;
+#pragma unroll
+      for (int k = 0; k < (NV + LPR - 1) / LPR; ++k) {
+        const int e = el + k * LPR * W;
+        if (e >= e0 && e < e1 && CCC_IN_BOUNDS(pair + e / SS, args.out_len, args.status)) {
+          const Vec t = *reinterpret_cast<const Vec *>(src + e);
+          if constexpr (W == 4)
+            stcs4(dst + e, t.x);
+          else
+            __stcs(dst + e, t.x[0]);
         }
-        // 4 n_ij = sum over the pair's table: the row sums of SNP i's s lanes.
-        int32_t n4 = 0;
-#pragma unroll
-        for (int k = 0; k < S; ++k) n4 += __shfl_sync(0xffffffffu, rs, src0 + k);
-        int32_t colsum[S];
-        if (want_ccc && !persnp) {
-#pragma unroll
-          for (int b = 0; b < S; ++b) {
-            colsum[b] = 0;
-#pragma unroll
-            for (int k = 0; k < S; ++k) colsum[b] += __shfl_sync(0xffffffffu, r[b], src0 + k);
-          }
-        }
-        if (!(row_ok && i < j && j < n_v && i >= args.i_begin && i < args.i_end)) continue;
-        if (!CCC_IN_BOUNDS(row_base + j - args.pair0, args.out_len, args.status)) continue;
-        const int64_t base = (row_base + j - args.pair0) * (S * S) + a * S;
-        store_row<S>(args.tally + base, r);
-        if (!want_ccc) continue;
-        float cv[S];
-        const float d = n4 == 0 ? 1.f : static_cast<float>(n4);
-        const float inv = rcp_count(d);
-        if (persnp) {
-          const float *wjs = stage + ((c - cb) * PW + jl) * S;
-#pragma unroll
-          for (int b = 0; b < S; ++b)
-            cv[b] = __fmul_rn(__fmul_rn(__fmul_rn(static_cast<float>(r[b]), inv), wi), wjs[b]);
-        } else {
-          const float wia = joint_factor(static_cast<float>(rs), d, inv, args.gamma);
-#pragma unroll
-          for (int b = 0; b < S; ++b) {
-            const float wjb = joint_factor(static_cast<float>(colsum[b]), d, inv, args.gamma);
-            cv[b] = __fmul_rn(__fmul_rn(div_count(static_cast<float>(r[b]), d, inv), wia), wjb);
-          }
-        }
-        store_row<S>(args.ccc + base, cv);
       }
     }
+  }
+  __device__ __forceinline__ static void stcs4(int *dst, const int (&x)[4]) {
+    __stcs(reinterpret_cast<int4 *>(dst), make_int4(x[0], x[1], x[2], x[3]));
+  }
+  __device__ __forceinline__ static void stcs4(float *dst, const float (&x)[4]) {
+    __stcs(reinterpret_cast<float4 *>(dst), make_float4(x[0], x[1], x[2], x[3]));
   }
 };
 
@@ -260,8 +394,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMultiThreads, 1)
       maps.m, sp, args, nkb, args.status);
 }
 
+template <int S>
 constexpr size_t multi_fp4_smem() {
-  return tcp::smem_bytes_nb(kMultiRectNB, kMultiEpiWarps, EpiMultiT<2, kMultiRectQ>::STAGE_BYTES_PER_WARP);
+  return tcp::smem_bytes_nb(kMultiRectNB, kMultiEpiWarps, EpiMultiT<S, kMultiRectQ>::STAGE_BYTES_PER_WARP);
 }
 constexpr size_t multi_smem() {
   return tcp::smem_bytes(kMultiEpiWarps, EpiMultiT<2, 8>::STAGE_BYTES_PER_WARP);
@@ -344,7 +479,7 @@ int launch_tally2_multi_fp4_s(const MultiMaps &maps, const MultiArgs &a, int gro
   int &max_clusters = max_clusters_dev[dev_c];
   if (max_clusters == 0) {
     if (cudaFuncSetAttribute(k_tally2_multi_fp4<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(multi_fp4_smem())) != cudaSuccess)
+                             static_cast<int>(multi_fp4_smem<S>())) != cudaSuccess)
       return CCC_ECUDA;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr;
@@ -354,7 +489,7 @@ int launch_tally2_multi_fp4_s(const MultiMaps &maps, const MultiArgs &a, int gro
     attr.val.clusterDim.z = 1;
     cfg.gridDim = dim3(static_cast<unsigned>(num_sms), 1, 1);
     cfg.blockDim = dim3(kMultiThreads, 1, 1);
-    cfg.dynamicSmemBytes = multi_fp4_smem();
+    cfg.dynamicSmemBytes = multi_fp4_smem<S>();
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     int n = 0;
@@ -363,7 +498,7 @@ int launch_tally2_multi_fp4_s(const MultiMaps &maps, const MultiArgs &a, int gro
     max_clusters = n < num_sms / 2 ? n : num_sms / 2;
   }
   const int64_t clusters = tiles < max_clusters ? tiles : max_clusters;
-  k_tally2_multi_fp4<S><<<static_cast<unsigned>(2 * clusters), kMultiThreads, multi_fp4_smem(),
+  k_tally2_multi_fp4<S><<<static_cast<unsigned>(2 * clusters), kMultiThreads, multi_fp4_smem<S>(),
                           s>>>(maps, a, sp, nkb);
   return note_launch();
 }
