@@ -77,7 +77,8 @@ struct EpiMultiT {
   using Params = MultiArgs;
   static constexpr int PW = snps_per_quarter(S);
   static constexpr int CHUNKS = NBQ / 2;  // of a warp
-  // FP4 tiles with S = 2 or odd S: the outputs leave through shared memory
+  // FP4 tiles with S = 2 or odd S, e4m3 tiles with odd S <= 13 (15 does not fit
+  // beside the operand stages, 2 neither): the outputs leave through shared memory
   // (put_chunk).  Otherwise (direct) a lane stores its own row of the table in
   // pieces of 16 bytes (S = 4, 8) or 8 (S = 6), which make up runs of S^2 words
   // anyway; the stage's traffic then costs more than it saves, because it
@@ -85,16 +86,21 @@ struct EpiMultiT {
   //   S = 4, 10,000 x 16,384: 4536 / 4751; 3,000 x 4,000: 159 / 217
   //   S = 8, 2,000 x 8,000: 460 / 447; 3,000 x 2,000, JOINT: 668 / 824
   //   S = 6, 3,000 x 4,000: 487 / 461; 3,000 x 1,500, JOINT: 455 / 551
-  // The e4m3 tiles' operand stages leave no room for it.  Loading all of a warp's
-  // chunks and releasing the accumulator before the first is stored was slower
-  // for every S (S = 4, 10,000 x 16,384: 4601; S = 3, 3,000 x 4,000: 175 for 168).
-  static constexpr bool STAGED = NBQ == kMultiRectQ && (S == 2 || S % 2 == 1);
+  // e4m3, JOINT, the sums over columns bound S > 7 at short K and the stage costs a
+  // little there (S = 9, 2,000 x 1,500: 711 / 719; S = 11, 1,500 x 1,500: 657 / 761),
+  // but at long K direct stores delay the operand loads (S = 11, 1,500 x 16,384:
+  // 2744 / 2463; S = 13, 1,200 x 16,384: 1965 / 1661).
+  // Loading all of a warp's chunks and releasing the accumulator before the first
+  // is stored was slower for every S (S = 4, 10,000 x 16,384: 4601; S = 3, 3,000 x
+  // 4,000: 175 for 168).
+  static constexpr bool STAGED = NBQ == kMultiRectQ ? S == 2 || S % 2 == 1 : S % 2 == 1 && S <= 13;
   // A marker i's words of one chunk, RUN = PW S^2, start RUN_LD words apart:
   // RUN_LD = S^2 (mod 32), so that the rows that the lanes (u, a) write at
-  // u RUN_LD + a S fall on different banks.
+  // u RUN_LD + a S fall on different banks (e4m3, S = 3: as near to it as fits).
   static constexpr int SS = S * S;
   static constexpr int RUN = PW * SS;
-  static constexpr int RUN_LD = SS % 32 + (RUN - SS % 32 + 31) / 32 * 32;
+  static constexpr int RUN_LD =
+      NBQ == 8 && S == 3 ? 91 : SS % 32 + (RUN - SS % 32 + 31) / 32 * 32;
   static constexpr int W = S % 2 == 0 ? 4 : 1;  // words a lane stores
   static constexpr int NV = RUN / W;
   static constexpr int LPR = NV <= 16 ? 16 : 32;  // lanes of a run
@@ -271,6 +277,8 @@ struct EpiMultiT {
   // GB300, 3,000 markers, us per call, direct -> staged:
   //   4,000 individuals:  S = 2: 98 -> 85, 3: 235 -> 168, 5 (JOINT): 504 -> 426, 7: 979 -> 674
   //   16,384 individuals: S = 2: 174 -> 171, 3: 340 -> 338, 5: 977 -> 880, 7: 1984 -> 1744
+  // e4m3, 4,096 individuals: 2,000 markers, S = 9: 1035 -> 628; 1,500, S = 11: 1029 -> 719;
+  //   1,200, S = 13: 922 -> 487; 4,000, S = 3: 461 -> 322
   template <typename T>
   __device__ __forceinline__ static void put_chunk(const MultiArgs &args, int64_t i0, int64_t j0,
                                                    int lane, const T *stage, T *out) {
@@ -398,8 +406,11 @@ template <int S>
 constexpr size_t multi_fp4_smem() {
   return tcp::smem_bytes_nb(kMultiRectNB, kMultiEpiWarps, EpiMultiT<S, kMultiRectQ>::STAGE_BYTES_PER_WARP);
 }
+template <int S>
 constexpr size_t multi_smem() {
-  return tcp::smem_bytes(kMultiEpiWarps, EpiMultiT<2, 8>::STAGE_BYTES_PER_WARP);
+  static_assert(tcp::smem_bytes(kMultiEpiWarps, EpiMultiT<S, 8>::STAGE_BYTES_PER_WARP) <= 232448,
+                "dynamic shared memory limit");
+  return tcp::smem_bytes(kMultiEpiWarps, EpiMultiT<S, 8>::STAGE_BYTES_PER_WARP);
 }
 
 // Persistent grid size for a pair kernel of kMultiThreads threads.
@@ -527,7 +538,7 @@ int launch_tally2_multi_s(const CUtensorMap &tm, const MultiArgs &a, int64_t nB,
   int &max_clusters = max_clusters_dev[dev_c];
   if (max_clusters == 0) {
     if (cudaFuncSetAttribute(k_tally2_multi<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(multi_smem())) != cudaSuccess)
+                             static_cast<int>(multi_smem<S>())) != cudaSuccess)
       return CCC_ECUDA;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr;
@@ -537,7 +548,7 @@ int launch_tally2_multi_s(const CUtensorMap &tm, const MultiArgs &a, int64_t nB,
     attr.val.clusterDim.z = 1;
     cfg.gridDim = dim3(static_cast<unsigned>(num_sms), 1, 1);
     cfg.blockDim = dim3(kMultiThreads, 1, 1);
-    cfg.dynamicSmemBytes = multi_smem();
+    cfg.dynamicSmemBytes = multi_smem<S>();
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     int n = 0;
@@ -546,7 +557,7 @@ int launch_tally2_multi_s(const CUtensorMap &tm, const MultiArgs &a, int64_t nB,
     max_clusters = n < num_sms / 2 ? n : num_sms / 2;
   }
   const int64_t clusters = tiles < max_clusters ? tiles : max_clusters;
-  k_tally2_multi<S><<<static_cast<unsigned>(2 * clusters), kMultiThreads, multi_smem(), s>>>(tm, a, sp,
+  k_tally2_multi<S><<<static_cast<unsigned>(2 * clusters), kMultiThreads, multi_smem<S>(), s>>>(tm, a, sp,
                                                                                           nkb);
   return note_launch();
 }

@@ -45,10 +45,12 @@ def test_rows_and_factors(s, n_f):
         assert_ccc_close(c, ec, what=f"s={s} n_f={n_f}")
 
 
-@pytest.mark.parametrize("s", [2, 3, 5, 7])
+# (s, operand): FP4 and e4m3 (1) tiles; more than eight states are e4m3 by themselves.
+@pytest.mark.parametrize("s,operand", [(2, 0), (3, 0), (5, 0), (7, 0), (3, 1), (5, 1), (7, 1),
+                                       (9, 0), (11, 0), (13, 0)])
 @pytest.mark.parametrize("dv", [-1, 0, 1])
 @pytest.mark.parametrize("norm", [0, 1])
-def test_staged_outputs(s, dv, norm):
+def test_staged_outputs(s, operand, dv, norm):
     """Outputs stored as runs (S = 2 and odd S): nothing outside the pairs of the call."""
     import torch
 
@@ -60,10 +62,10 @@ def test_staged_outputs(s, dv, norm):
     lo, hi = rng.integers(0, s + 1, size=(2, n_v, 112), dtype=np.uint8)
     g = (lo | (hi << 4)).astype(np.uint8)
     dev = to_device_bytes(g)
-    opts = ccc.ccc_opts_default(norm=norm)
+    opts = ccc.ccc_opts_default(norm=norm, operand=operand)
     opts.split = 1
     ws = workspace(ccc.ccc_multi_workspace_size(dev, n_f, s, opts))
-    opts = ccc.ccc_opts_default(norm=norm, workspace=ws)
+    opts = ccc.ccc_opts_default(norm=norm, workspace=ws, operand=operand)
     opts.split = 1
     guard = 64
     inner = slice(guard, guard + npairs * ss)
