@@ -77,10 +77,10 @@ struct EpiMultiT {
   using Params = MultiArgs;
   static constexpr int PW = snps_per_quarter(S);
   static constexpr int CHUNKS = NBQ / 2;  // of a warp
-  // FP4 tiles with S = 2 or odd S, e4m3 tiles with odd S <= 13 (15 does not fit
-  // beside the operand stages, 2 neither): the outputs leave through shared memory
+  // FP4 tiles with S = 2 or odd S, e4m3 tiles with odd S, 10 or 14 (S = 2
+  // does not fit beside their operand stages): the outputs leave through shared memory
   // (put_chunk).  Otherwise (direct) a lane stores its own row of the table in
-  // pieces of 16 bytes (S = 4, 8) or 8 (S = 6), which make up runs of S^2 words
+  // pieces of 16 bytes (S = 4, 8, 12) or 8 (S = 6), which make up runs of S^2 words
   // anyway; the stage's traffic then costs more than it saves, because it
   // competes with the MMAs' operand reads.  GB300, us per call, direct / staged:
   //   S = 4, 10,000 x 16,384: 4536 / 4751; 3,000 x 4,000: 159 / 217
@@ -89,18 +89,19 @@ struct EpiMultiT {
   // e4m3, JOINT, the sums over columns bound S > 7 at short K and the stage costs a
   // little there (S = 9, 2,000 x 1,500: 711 / 719; S = 11, 1,500 x 1,500: 657 / 761),
   // but at long K direct stores delay the operand loads (S = 11, 1,500 x 16,384:
-  // 2744 / 2463; S = 13, 1,200 x 16,384: 1965 / 1661).
+  // 2744 / 2463; S = 13, 1,200 x 16,384: 1965 / 1661; S = 10, 1,500 x 1,500: 392 /
+  // 423, x 16,384: 1266 / 1190; S = 15, 1,200 x 16,384: 2291 / 1738).
   // Loading all of a warp's chunks and releasing the accumulator before the first
   // is stored was slower for every S (S = 4, 10,000 x 16,384: 4601; S = 3, 3,000 x
   // 4,000: 175 for 168).
-  static constexpr bool STAGED = NBQ == kMultiRectQ ? S == 2 || S % 2 == 1 : S % 2 == 1 && S <= 13;
+  static constexpr bool STAGED = NBQ == kMultiRectQ ? S == 2 || S % 2 == 1 : S % 2 == 1 || S == 10 || S == 14;
   // A marker i's words of one chunk, RUN = PW S^2, start RUN_LD words apart:
   // RUN_LD = S^2 (mod 32), so that the rows that the lanes (u, a) write at
-  // u RUN_LD + a S fall on different banks (e4m3, S = 3: as near to it as fits).
+  // u RUN_LD + a S fall on different banks (S = 3 on e4m3 tiles, 10, 15: as near to it as fits).
   static constexpr int SS = S * S;
   static constexpr int RUN = PW * SS;
   static constexpr int RUN_LD =
-      NBQ == 8 && S == 3 ? 91 : SS % 32 + (RUN - SS % 32 + 31) / 32 * 32;
+      NBQ == 8 && S == 3 ? 91 : S == 10 ? 308 : S == 15 ? 464 : SS % 32 + (RUN - SS % 32 + 31) / 32 * 32;
   static constexpr int W = S % 2 == 0 ? 4 : 1;  // words a lane stores
   static constexpr int NV = RUN / W;
   static constexpr int LPR = NV <= 16 ? 16 : 32;  // lanes of a run
@@ -270,15 +271,15 @@ struct EpiMultiT {
 
   // One chunk of one array from the stage to global memory.  For each of the
   // warp's markers i the words of the pairs (i, j0 .. j0 + PW - 1) are contiguous
-  // there, so the lanes store them side by side: 16 bytes each for S = 2 (a
-  // pair's 4 words are one 16-byte unit), words for odd S.  When each
+  // there, so the lanes store them side by side: 16 bytes each for even S (a
+  // pair's S^2 words are then whole 16-byte units), words for odd S.  When each
   // lane stored its own row of the table, an instruction wrote 32 pieces of at
   // most 8 bytes in as many 128-byte lines as the warp has markers.
   // GB300, 3,000 markers, us per call, direct -> staged:
   //   4,000 individuals:  S = 2: 98 -> 85, 3: 235 -> 168, 5 (JOINT): 504 -> 426, 7: 979 -> 674
   //   16,384 individuals: S = 2: 174 -> 171, 3: 340 -> 338, 5: 977 -> 880, 7: 1984 -> 1744
   // e4m3, 4,096 individuals: 2,000 markers, S = 9: 1035 -> 628; 1,500, S = 11: 1029 -> 719;
-  //   1,200, S = 13: 922 -> 487; 4,000, S = 3: 461 -> 322
+  //   1,200, S = 13: 922 -> 487, S = 14: 706 -> 493, S = 15: 1487 -> 533; 4,000, S = 3: 461 -> 322
   template <typename T>
   __device__ __forceinline__ static void put_chunk(const MultiArgs &args, int64_t i0, int64_t j0,
                                                    int lane, const T *stage, T *out) {

@@ -47,7 +47,8 @@ def test_rows_and_factors(s, n_f):
 
 # (s, operand): FP4 and e4m3 (1) tiles; more than eight states are e4m3 by themselves.
 @pytest.mark.parametrize("s,operand", [(2, 0), (3, 0), (5, 0), (7, 0), (3, 1), (5, 1), (7, 1),
-                                       (9, 0), (11, 0), (13, 0)])
+                                       (9, 0), (10, 0), (11, 0), (13, 0),
+                                       (14, 0), (15, 0)])
 @pytest.mark.parametrize("dv", [-1, 0, 1])
 @pytest.mark.parametrize("norm", [0, 1])
 def test_staged_outputs(s, operand, dv, norm):
