@@ -501,12 +501,15 @@ struct PairMaps {
 //     max_b r_ab w_j(b) w_i(a) > threshold 4 n_ij,
 // and n_ij >= n_i + n_j - n_f (the entries that either SNP misses), so a row with
 //     max_b r_ab w_j(b) < R (n_i - n_f) + R n_j,   R = 4 threshold / w_i(a)
-// (less 2^-16 for the roundings) holds no hit.  At 1% missing entries the two
-// sides of n_ij differ by 10^-4, so few more rows pass than have to; the 16 j of
-// a warp in which one does go through the exact test (filter_cols), and the hit
-// list is what Epi2 produces.  Per warp and tile about 450 instructions instead
-// of 1,600.  GB300, 50,000 x 4,096: 6.74 -> 6.12 ms per call
-// (5.79 with no test at all).
+// (less 2^-16 for the roundings) holds no hit.  The two terms of the bound may
+// cancel to less than the rounding of the first one (SNPs typed on individuals
+// that hardly overlap), so that one is rounded down: what the sum then errs
+// upwards is a fraction of itself.  At 1% missing entries the two sides of n_ij
+// differ by 10^-4, so few more rows pass than have to; the 16 j of a warp in
+// which one does go through the exact test (filter_cols), and the hit list is
+// what Epi2 produces.  Per warp and tile about 450 instructions instead of
+// 1,600.  GB300, 50,000 x 4,096: 6.74 -> 6.12 ms per call (5.79 with no test at
+// all).
 struct Epi2Rect {
   using Params = Tally2Args;
   using Sched = RectSchedT<128, kRectJ, kRectNB>;
@@ -591,7 +594,7 @@ struct Epi2Rect {
     // JOINT, and thresholds that empty tables pass, go to the exact test at once.
     const bool first = persnp && args.threshold > 0.f;
     const float R = 4.f * (1.f - 0x1p-16f) * args.threshold / (a ? wi1 : wi0);
-    const float base = rowok ? R * static_cast<float>(e.ni - static_cast<int32_t>(args.n_f))
+    const float base = rowok ? __fmul_rd(R, static_cast<float>(e.ni - static_cast<int32_t>(args.n_f)))
                              : __int_as_float(0x7f800000);
     float4 *const js = reinterpret_cast<float4 *>(stage);
     __syncwarp();  // the previous tile's reads are done
