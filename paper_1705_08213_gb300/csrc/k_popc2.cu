@@ -34,6 +34,7 @@
 #include "ccc_dev.cuh"
 #include "ccc_launch.h"
 #include "ccc_metric.cuh"
+#include "popc_tiles.cuh"
 
 namespace ccc {
 namespace {
@@ -42,19 +43,6 @@ constexpr int TS = 32;       // SNPs per tile side
 constexpr int KC = 8;        // 64-entry words per stage
 constexpr int THREADS = 256;
 constexpr int LDS = TS + 1;  // padded row (u64) against bank conflicts
-
-__device__ __forceinline__ void tile_coords(int64_t t, int64_t nB, int64_t &I, int64_t &J) {
-  // Row-major upper triangle with diagonal: row I holds nB - I tiles.
-  const double b = 2.0 * nB + 1.0;
-  int64_t r = static_cast<int64_t>((b - sqrt(b * b - 8.0 * static_cast<double>(t))) * 0.5);
-  if (r < 0) r = 0;
-  if (r >= nB) r = nB - 1;
-  auto start = [&](int64_t row) { return row * nB - row * (row - 1) / 2; };
-  while (r > 0 && start(r) > t) --r;
-  while (r + 1 < nB && start(r + 1) <= t) ++r;
-  I = r;
-  J = r + (t - start(r));
-}
 
 // Planes H, A, M of 32 SNPs x KC words, 2 halves of 16 bytes per word.
 __device__ __forceinline__ void load_stage(const uint64_t *__restrict__ planes, int64_t w64,
@@ -136,7 +124,7 @@ __global__ void __launch_bounds__(THREADS, 2)
   __shared__ uint64_t sI[3][KC][LDS];
   __shared__ uint64_t sJ[3][KC][LDS];
   int64_t I, J;
-  tile_coords(t0 + blockIdx.x, nB, I, J);
+  PopcTri{nB}.coords(t0 + blockIdx.x, I, J);
   const int64_t n_v = args.n_v;
   const int tx = threadIdx.x & 15;
   const int ty = threadIdx.x >> 4;
@@ -252,14 +240,10 @@ int64_t popc2_tiles(int64_t n_v) {
 int launch_tally2_popc(const Tally2Args &a, const uint64_t *planes, int64_t w64, cudaStream_t s,
                        int split) {
   const int64_t nB = (a.n_v + TS - 1) / TS;
-  // Row blocks [B0, B1) of the phase; tiles before row B are B nB - B (B - 1) / 2.
-  const int64_t B0 = (a.i_begin > 0 ? a.i_begin : 0) / TS;
-  const int64_t B1 = a.i_end < a.n_v ? (a.i_end + TS - 1) / TS : nB;
-  auto start = [&](int64_t r) { return r * nB - r * (r - 1) / 2; };
-  const int64_t t0 = start(B0);
-  const int64_t tiles = start(B1) - t0;
+  int64_t t0;
+  const int64_t tiles = PopcTri::in_rows(a.n_v, a.i_begin, a.i_end, TS, &t0);
   if (tiles <= 0) return CCC_OK;
-  if (tiles > 0x7fffffffLL) return CCC_ERANGE;
+  if (!popc_in_range(a.n_v, a.i_begin, a.i_end)) return CCC_ERANGE;
   // Parts of whole KC-word stages; split > 1 only with a.tally zeroed, no
   // thresholded output and the CCC values formed afterwards.
   const int64_t stages = (w64 + KC - 1) / KC;
@@ -267,9 +251,11 @@ int launch_tally2_popc(const Tally2Args &a, const uint64_t *planes, int64_t w64,
   if (split > stages) split = static_cast<int>(stages);
   const int64_t part_words = (stages + split - 1) / split * KC;
   const int parts = static_cast<int>((w64 + part_words - 1) / part_words);
-  const dim3 grid(static_cast<unsigned>(tiles), static_cast<unsigned>(parts > 0 ? parts : 1), 1);
-  k_tally2_popc<<<grid, THREADS, 0, s>>>(planes, w64, a, nB, t0, parts > 1 ? part_words : w64);
-  return note_launch();
+  return popc_launches(t0, tiles, [&](int64_t first, int64_t count) {
+    const dim3 grid(static_cast<unsigned>(count), static_cast<unsigned>(parts > 0 ? parts : 1), 1);
+    k_tally2_popc<<<grid, THREADS, 0, s>>>(planes, w64, a, nB, first, parts > 1 ? part_words : w64);
+    return note_launch();
+  });
 }
 
 int launch_metric2(const int32_t *tally, const float *w, int64_t n_v, float gamma, int32_t norm,
