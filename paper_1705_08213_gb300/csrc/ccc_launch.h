@@ -111,9 +111,6 @@ struct Tally2Args {
   // SM-pair kernels: tallies below 2^16 stored as four 16-bit numbers per pair
   // (8 bytes, tally an array of them; no CCC values).
   bool pack16 = false;
-  // Cycles between the output lines of a tile in the SM-pair kernels (set by
-  // their launches; 0 = stored as fast as they come).
-  uint32_t pace = 0;
   // Row range of a phase: only pairs with i_begin <= i < i_end are computed and
   // pair (i, j) is stored at index pair_index(i, j) - pair0.
   int64_t i_begin = 0;

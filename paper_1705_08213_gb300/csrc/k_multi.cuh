@@ -120,7 +120,7 @@ struct EpiMultiT {
   template <int NC, bool PRELOAD = false>
   __device__ static void tile(const Params &args, const Sched &sc, int rank, int quarter,
                               int lane, uint32_t t_base, uint32_t release_cluster_bar, int c0,
-                              float *stage, tcp::NoEarly, bool) {
+                              float *stage, tcp::NoEarly, int) {
     static_assert(!PRELOAD, "s-state tiles run on the two-accumulator pipeline");
     static_assert(NBQ % 2 == 0, "two column halves");
     const int cb = (c0 / NC) * CHUNKS;
@@ -336,7 +336,7 @@ struct EpiMultiSplit {
   template <int NC, bool PRELOAD = false>
   __device__ static void tile(const Params &args, const SplitSchedPair &sc, int rank, int quarter,
                               int lane, uint32_t t_base, uint32_t release_cluster_bar, int c0,
-                              float *, tcp::NoEarly, bool) {
+                              float *, tcp::NoEarly, int) {
     static_assert(!PRELOAD, "s-state tiles run on the two-accumulator pipeline");
     const int u = lane / S;
     const int a = lane - u * S;

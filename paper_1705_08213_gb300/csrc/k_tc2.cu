@@ -194,17 +194,18 @@ struct Epi2Staged {
   // table r_ik of the 3-way classes; args.pack16), a line being 64 bytes.
   enum Mode { TALLY, PACK16, PERSNP, JOINT };
 
-  // Cycles from line to line that spread a tile's lines (2 NC + 1, NC = 32 / ew
-  // chunks per warp) over about 4/5 of the MMAs of the next tile, K stages of
-  // about 640 (e2m1) or 560 (e4m3) cycles; kLineCycles is what a line's stores
+  // Cycles from line to line that spread a tile's lines (2 NC + 1, NC = 32 / EW
+  // chunks per warp) over about 4/5 of the MMAs of the cluster's next tile, k_next
+  // K stages of about 640 (e2m1) or 560 (e4m3) cycles (0: no next tile, stored as
+  // they come); kLineCycles is what a line's stores
   // take by themselves.  20,000 SNPs, all panels' tiles in lockstep: stored as
   // they come, the burst of each tile's 512 KB delays the operand loads
   // (16,384 individuals 3.89 ms, 8,192 2.45 ms, 4,096 1.67 ms); spread, and the
   // warps one after another, 3.62, 2.25 and 1.60 ms.
   static constexpr uint32_t kLineCycles = 600;
-  static uint32_t pace(int stages, bool fp4, int ew) {
-    return static_cast<uint32_t>(stages) * (fp4 ? 640u : 560u) * 4u / 5u /
-           static_cast<uint32_t>(64 / ew + 1);
+  template <int EW, bool FP4>
+  __device__ __forceinline__ static uint32_t pace(int k_next) {
+    return static_cast<uint32_t>(k_next) * (FP4 ? 640u : 560u) * 4u / 5u / (64u / EW + 1u);
   }
 
   // PERSNP factors of a tile, loaded during the one before: inside the tile a
@@ -237,16 +238,16 @@ struct Epi2Staged {
   __device__ __forceinline__ static void body(const Tally2Args &args, Tile2 sc, int quarter,
                                               int lane, uint32_t t_base,
                                               uint32_t release_cluster_bar, int c0, float *stage,
-                                              const Early<NC> &e, bool more) {
+                                              const Early<NC> &e, int k_next) {
     if (args.pack16)
       run<NC, PRELOAD, PACK16>(args, sc, quarter, lane, t_base, release_cluster_bar, c0, stage, e,
-                               more);
+                               k_next);
     else if (args.ccc == nullptr)
-      run<NC, PRELOAD, TALLY>(args, sc, quarter, lane, t_base, release_cluster_bar, c0, stage, e, more);
+      run<NC, PRELOAD, TALLY>(args, sc, quarter, lane, t_base, release_cluster_bar, c0, stage, e, k_next);
     else if (args.norm == CCC_NORM_PERSNP)
-      run<NC, PRELOAD, PERSNP>(args, sc, quarter, lane, t_base, release_cluster_bar, c0, stage, e, more);
+      run<NC, PRELOAD, PERSNP>(args, sc, quarter, lane, t_base, release_cluster_bar, c0, stage, e, k_next);
     else
-      run<NC, PRELOAD, JOINT>(args, sc, quarter, lane, t_base, release_cluster_bar, c0, stage, e, more);
+      run<NC, PRELOAD, JOINT>(args, sc, quarter, lane, t_base, release_cluster_bar, c0, stage, e, k_next);
   }
 
   // The lane's four SNPs i of a tile.
@@ -339,7 +340,7 @@ struct Epi2Staged {
   __device__ __forceinline__ static void run(const Tally2Args &args, Tile2 sc, int quarter,
                                              int lane, uint32_t t_base,
                                              uint32_t release_cluster_bar, int c0, float *stage,
-                                             const Early<NC> &e, bool more) {
+                                             const Early<NC> &e, int k_next) {
     constexpr int EW = 32 / NC;
     const int ew = c0 / NC * 4 + quarter;
     char *const ring = reinterpret_cast<char *>(stage);
@@ -371,7 +372,7 @@ struct Epi2Staged {
     // Line q starts no earlier than q pace cycles after the first, and the
     // warps' first lines one after another (in an order of the cluster's own),
     // where the next tile's MMAs leave time for it.
-    const uint32_t pace = more ? args.pace : 0u;
+    const uint32_t pace = Epi2Staged::pace<EW, PRELOAD>(k_next);
     const uint32_t turn = (static_cast<uint32_t>(ew) + (blockIdx.x >> 1)) % EW;
     const uint32_t begin = static_cast<uint32_t>(clock()) +
                            (pace > kLineCycles ? (pace - kLineCycles) / EW * turn : 0u);
@@ -431,13 +432,13 @@ struct Epi2Pair {
   template <int NC, bool PRELOAD = false>
   __device__ static void tile(const Params &args, const TriSchedPair &sc, int rank, int quarter,
                               int lane, uint32_t t_base, uint32_t release_cluster_bar, int c0,
-                              float *stage, const Epi2Staged::Early<NC> &e, bool more) {
+                              float *stage, const Epi2Staged::Early<NC> &e, int k_next) {
     if (args.hits != nullptr)  // thresholded output stores little: no staging
       Epi2::body<NC, true, PRELOAD>(args, Tile2{2 * sc.I + rank, sc.J}, quarter, lane, t_base,
                                     release_cluster_bar, c0);
     else
       Epi2Staged::body<NC, PRELOAD>(args, Tile2{2 * sc.I + rank, sc.J}, quarter, lane, t_base,
-                                    release_cluster_bar, c0, stage, e, more);
+                                    release_cluster_bar, c0, stage, e, k_next);
   }
 };
 
@@ -547,7 +548,7 @@ struct Epi2Rect {
   template <int NC, bool PRELOAD>
   __device__ static void tile(const Params &args, const Sched &sc, int rank, int quarter, int lane,
                               uint32_t t_base, uint32_t release_cluster_bar, int c0,
-                              float *stage, const Early &e, bool) {
+                              float *stage, const Early &e, int) {
     static_assert(!PRELOAD, "two accumulators: each warp releases after its last load");
     const int half = c0 / NC;
     const int64_t ib = static_cast<int64_t>(2 * sc.I + rank) * SNP_I;  // the CTA's first SNP i
@@ -735,7 +736,7 @@ struct Epi2Split {
   template <int NC, bool PRELOAD = false>
   __device__ static void tile(const Params &args, const SplitSchedPair &sc, int rank, int quarter,
                               int lane, uint32_t t_base, uint32_t release_cluster_bar, int c0,
-                              float *, tcp::NoEarly, bool) {
+                              float *, tcp::NoEarly, int) {
     body<NC, PRELOAD>(args, Tile2{2 * sc.I + rank, sc.J}, quarter, lane, t_base,
                       release_cluster_bar, c0);
   }
@@ -918,14 +919,14 @@ struct EpiBatchPair {
   template <int NC, bool PRELOAD = false>
   __device__ static void tile(const Params &bp, const BatchSchedPair &sc, int rank, int quarter,
                               int lane, uint32_t t_base, uint32_t release_cluster_bar, int c0,
-                              float *stage, const Epi2Staged::Early<NC> &e, bool more) {
+                              float *stage, const Epi2Staged::Early<NC> &e, int k_next) {
     const BatchPanel &q = bp.p[sc.p];
     if (q.split > 1)  // a K part: partial tallies added into the zeroed output
       Epi2Split::body<NC, PRELOAD>(q.args, Tile2{2 * sc.t.I + rank, sc.t.J}, quarter, lane, t_base,
                                    release_cluster_bar, c0);
     else
       Epi2Staged::body<NC, PRELOAD>(q.args, Tile2{2 * sc.t.I + rank, sc.t.J}, quarter, lane,
-                                    t_base, release_cluster_bar, c0, stage, e, more);
+                                    t_base, release_cluster_bar, c0, stage, e, k_next);
   }
 };
 
@@ -1067,7 +1068,6 @@ int launch_tally2_tc_pair_batched(const Tally2Args *args, const uint8_t *const *
   }
   if (units == 0) return CCC_OK;
   const int ew = fp4 ? tcp::FP4_EW : epilogue_warps(static_cast<int>(kw / static_cast<double>(units)));
-  for (int k = 0; k < n; ++k) bp.p[k].args.pace = Epi2Staged::pace(bp.p[k].nkb, fp4, ew);
   static int max_clusters[kMaxDevices][3] = {};
   int &mc = max_clusters[dev][fp4 ? 2 : ew == 4 ? 0 : 1];
   if (mc == 0) {
@@ -1151,9 +1151,8 @@ int launch_tally2_tc_batched(const Tally2Args *args, const uint8_t *const *ops,
   return note_launch();
 }
 
-int launch_tally2_tc_pair(const Tally2Args &args, const uint8_t *op, int64_t rows_pad, int64_t kpad,
+int launch_tally2_tc_pair(const Tally2Args &a, const uint8_t *op, int64_t rows_pad, int64_t kpad,
                           int num_sms, cudaStream_t s, bool fp4) {
-  Tally2Args a = args;
   static bool attr_set[kMaxDevices] = {};
   const int dev = current_device();
   if (dev < 0) return CCC_ECUDA;
@@ -1224,7 +1223,6 @@ int launch_tally2_tc_pair(const Tally2Args &args, const uint8_t *op, int64_t row
   const int64_t tiles = tc2_pair_tiles(a.n_v, sp.I0, sp.I1);
   if (tiles == 0) return CCC_OK;
   const int ew = fp4 ? tcp::FP4_EW : epilogue_warps(nkb);
-  a.pace = Epi2Staged::pace(nkb, fp4, ew);
   // Persistent grid: as many SM pairs as can be resident at once.
   int &mc = max_clusters[dev][fp4 ? 2 : ew == 4 ? 0 : 1];
   if (mc == 0) {

@@ -207,8 +207,8 @@ struct NoEarly {};
 //        from global memory, loaded ahead of it (tile: there is one);
 //      template <int NC> static void tile(const Params&, const Sched&, int rank,
 //        int quarter, int lane, uint32_t t_base, uint32_t release_cluster_bar,
-//        int c0, float *stage, const T&, bool more); the release arrives at a
-//        cluster address; more: the cluster has another tile after this one;
+//        int c0, float *stage, const T&, int k_next); the release arrives at a
+//        cluster address; k_next: K stages of the cluster's next tile (0: none);
 //        static constexpr int STAGE_BYTES_PER_WARP: shared memory each epilogue
 //        warp may use at `stage` (the kernel is launched with
 //        smem_bytes(EW, STAGE_BYTES_PER_WARP)), slice 4 (c0 / NC) + quarter.
@@ -440,7 +440,7 @@ __device__ __forceinline__ void persistent_gemm_pair(const CUtensorMap *tm,
                                         map_to_rank(tempty_bar(acc), 0), c0,
                                         stage_base + (4 * half + quarter) *
                                                          (Epi::STAGE_BYTES_PER_WARP / 4),
-                                        early, next.valid);
+                                        early, next.valid ? next.k_blocks(nkb) : 0);
     }
   }
 
@@ -715,7 +715,7 @@ __device__ __forceinline__ void persistent_gemm_pair_packed(const CUtensorMap *t
       Epi::template tile<NC>(ep, sc, static_cast<int>(rank), quarter, lane, t_base,
                              map_to_rank(tempty_bar(acc), 0), c0,
                              stage_base + (4 * half + quarter) * (Epi::STAGE_BYTES_PER_WARP / 4),
-                             early, false);
+                             early, 0);
     }
   } else {
     // ---------------- converters (both CTAs)
