@@ -177,7 +177,8 @@ __global__ void __launch_bounds__(256) k_multi_unpack(const uint8_t *__restrict_
 // of byte q / 2 for even q), rows of kpad / 2 bytes (kpad a multiple of 256);
 // and, when w is set, the marker's PERSNP factors (the formula of
 // k_multi_counts) from the same read.  One 128-thread block per marker (markers
-// past n_v give zero rows, a quarter's last marker also its rows past S PW), a
+// past n_v give zero rows, a quarter's last marker also its rows past S PW), or,
+// without w, per marker and part of part_chunks 32-individual chunks of its row; a
 // thread 32 individuals at a time, eight of them per step:
 //   the low and high nibbles of eight entries are packed into one word each (x, y);
 //   an entry with x >= S or y >= S gets nibble 15 in both;
@@ -201,17 +202,19 @@ template <int S>
 __global__ void __launch_bounds__(128) k_multi_unpack_e2m1(const uint8_t *__restrict__ geno,
                                                            int64_t n_f, int64_t n_v, int64_t ld,
                                                            uint8_t *__restrict__ op, int64_t kpad,
-                                                           float *__restrict__ w, double gamma) {
+                                                           float *__restrict__ w, double gamma,
+                                                           int part_chunks) {
   constexpr int PW = snps_per_quarter(S);
   const int64_t i = blockIdx.x;
   const int u = static_cast<int>(i % PW);
   const int64_t row_bytes = kpad / 2;
   uint8_t *const rows = op + (32 * (i / PW) + S * u) * row_bytes;
   const uint8_t *const src = geno + i * ld;
-  const int chunks = static_cast<int>(kpad / 32);
+  const int begin = static_cast<int>(blockIdx.y) * part_chunks;
+  const int end = min(static_cast<int>(kpad / 32), begin + part_chunks);
   const int zeros = u == PW - 1 ? 32 - S * PW : 0;
   uint32_t c[S] = {}, n = 0;
-  for (int ch = threadIdx.x; ch < chunks; ch += 128) {
+  for (int ch = begin + threadIdx.x; ch < end; ch += 128) {
     const int64_t q0 = 32 * static_cast<int64_t>(ch);
     uint8_t *const dst = rows + 16 * ch;
     uint32_t in[8] = {};
@@ -372,8 +375,20 @@ int launch_multi_unpack(const uint8_t *geno, int64_t n_f, int64_t n_v, int64_t l
     const int64_t markers = quarters * snps_per_quarter(s);
     if (markers < 1) return CCC_OK;
     if (markers > 0x7FFFFFFFLL) return CCC_ERANGE;
+    // Without factors (tallies alone, JOINT) nothing is summed over a row, so few
+    // markers' rows are cut into parts of whole 4,096-individual steps, 16 blocks
+    // per SM in all.  GB300, us per call, a block per row / in parts (the call
+    // with factors, always a block per row): 100 x 1,000,000, s = 2: 1391 / 1219
+    // (1390), s = 8: 1565 / 1293 (1564); 40 x 300,000, s = 8: 476 / 382 (474);
+    // 300 x 16,384, s = 4: 41 / 39; 8 or 32 blocks per SM within 1%.
+    const int64_t chunks = kpad / 32, steps = (chunks + 127) / 128;
+    const int64_t want = w == nullptr ? (152 * 16 + markers - 1) / markers : 1;
+    const int64_t part_steps = (steps + want - 1) / want;
+    const int part_chunks = static_cast<int>(128 * part_steps);
+    const dim3 grid(static_cast<unsigned>(markers),
+                    static_cast<unsigned>((steps + part_steps - 1) / part_steps), 1);
     auto go = [&](auto kernel) {
-      kernel<<<static_cast<unsigned>(markers), 128, 0, st>>>(geno, n_f, n_v, ld, op, kpad, w, gamma);
+      kernel<<<grid, 128, 0, st>>>(geno, n_f, n_v, ld, op, kpad, w, gamma, part_chunks);
       return note_launch();
     };
     switch (s) {
