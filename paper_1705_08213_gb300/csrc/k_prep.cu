@@ -465,11 +465,14 @@ int launch_unpack_blocked(const uint64_t *geno, int64_t n_f, int64_t n_v, int64_
     return CCC_EINVAL;
   const int64_t nkb = kpad / kblock;
   if (snps_pad < 1 || nkb < 1) return CCC_OK;
-  // 32-SNP blocks times K ranges, about 32 blocks per SM in all.
+  // 32-SNP blocks times K ranges, about 32 blocks per SM in all, but no range
+  // shorter than the four K blocks whose loads a thread has in flight: shorter
+  // ones only add counts to be summed (1,000 x 30,000: 76.1 -> 71.0 us per call
+  // with ranges of one K block -> four; 512 x 1,000,000, ranges of 17: 315).
   const int64_t gx = snps_pad / 32;
   if (gx > 0x7FFFFFFF) return CCC_EINVAL;
   int64_t gy = (152 * 32 + gx - 1) / gx;
-  if (gy > nkb) gy = nkb;
+  if (gy > (nkb + 3) / 4) gy = (nkb + 3) / 4;
   if (gy > 65535) gy = 65535;
   const int64_t kb_per = (nkb + gy - 1) / gy;
   gy = (nkb + kb_per - 1) / kb_per;
