@@ -128,7 +128,8 @@ struct Layout {
   size_t op = 0;              // e4m3 operands [rows_pad][kpad] (TC path)
   size_t planes = 0;          // uint64 [n_v][w64][4] (POPC path)
   size_t lop = 0;             // masked 3-way operands (TC path)
-  size_t rtab = 0;            // int32 [pairs][4] 2-way tallies (3-way classes)
+  size_t rtab = 0;            // [pairs][4] 2-way tallies (3-way classes): int32, or 16-bit
+                              // numbers in its first half (tc3_class_table16)
   size_t cbuf = 0;            // compacted count rows per slab (3-way classes)
   size_t missing = 0;         // int32 [cbuf_slabs] missing entries of v_j
   size_t dscratch = 0;        // D counts of the wide class tiles in flight

@@ -91,6 +91,10 @@ struct EpiMultiT {
   // but at long K direct stores delay the operand loads (S = 11, 1,500 x 16,384:
   // 2744 / 2463; S = 13, 1,200 x 16,384: 1965 / 1661; S = 10, 1,500 x 1,500: 392 /
   // 423, x 16,384: 1266 / 1190; S = 15, 1,200 x 16,384: 2291 / 1738).
+  // The rule goes by S alone.  Against direct stores with IEEE divisions every S gains
+  // from the two together (S = 11, JOINT, 1,500 x 1,500: 1267 -> 761), but for e4m3 tiles
+  // with S = 6 or 8, PERSNP, around 4,000 individuals (2,500 x 4,000: 426 -> 434, 638 ->
+  // 649): the values come faster there and bunch the direct stores.
   // Loading all of a warp's chunks and releasing the accumulator before the first
   // is stored was slower for every S (S = 4, 10,000 x 16,384: 4601; S = 3, 3,000 x
   // 4,000: 175 for 168).

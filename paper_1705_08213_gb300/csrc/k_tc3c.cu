@@ -665,7 +665,7 @@ __device__ __forceinline__ int4 bits4(float4 v) {
 // 16-bit numbers are subtracted two at a time, and no value crosses lanes.
 // GB300, class kernels per call: 1,536 x 8,192 13.6 -> 11.4 ms (8.3 without its
 // stores, 7.9 without its loads either, 6.5 of MMAs); calls: 301 x 2,001 JOINT
-// 279 -> 213 us, 1,000 x 1,000 JOINT -> 2.95 ms (3.6 TB/s).
+// 279 -> 213 us (191 with k_gather3), 1,000 x 1,000 JOINT -> 2.95 ms (3.6 TB/s).
 template <int MODE>
 struct Epi3 {
   char *out[4];          // tally address of the lane's triple in the row's first lines
