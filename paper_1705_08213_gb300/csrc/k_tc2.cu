@@ -239,15 +239,16 @@ struct Epi2Staged {
                                               int lane, uint32_t t_base,
                                               uint32_t release_cluster_bar, int c0, float *stage,
                                               const Early<NC> &e, int k_next) {
-    if (args.pack16)
-      run<NC, PRELOAD, PACK16>(args, sc, quarter, lane, t_base, release_cluster_bar, c0, stage, e,
-                               k_next);
-    else if (args.ccc == nullptr)
-      run<NC, PRELOAD, TALLY>(args, sc, quarter, lane, t_base, release_cluster_bar, c0, stage, e, k_next);
-    else if (args.norm == CCC_NORM_PERSNP)
+    // In this order: the same code with PACK16 first, PERSNP after it, is laid out
+    // otherwise and takes 1.62 ms instead of 1.60 for 20,000 x 4,096.
+    if (args.ccc != nullptr && args.norm == CCC_NORM_PERSNP)
       run<NC, PRELOAD, PERSNP>(args, sc, quarter, lane, t_base, release_cluster_bar, c0, stage, e, k_next);
-    else
+    else if (args.ccc != nullptr)
       run<NC, PRELOAD, JOINT>(args, sc, quarter, lane, t_base, release_cluster_bar, c0, stage, e, k_next);
+    else if (args.pack16)
+      run<NC, PRELOAD, PACK16>(args, sc, quarter, lane, t_base, release_cluster_bar, c0, stage, e, k_next);
+    else
+      run<NC, PRELOAD, TALLY>(args, sc, quarter, lane, t_base, release_cluster_bar, c0, stage, e, k_next);
   }
 
   // The lane's four SNPs i of a tile.
@@ -433,20 +434,42 @@ struct Epi2Pair {
   __device__ static void tile(const Params &args, const TriSchedPair &sc, int rank, int quarter,
                               int lane, uint32_t t_base, uint32_t release_cluster_bar, int c0,
                               float *stage, const Epi2Staged::Early<NC> &e, int k_next) {
-    if (args.hits != nullptr)  // thresholded output stores little: no staging
-      Epi2::body<NC, true, PRELOAD>(args, Tile2{2 * sc.I + rank, sc.J}, quarter, lane, t_base,
-                                    release_cluster_bar, c0);
-    else
-      Epi2Staged::body<NC, PRELOAD>(args, Tile2{2 * sc.I + rank, sc.J}, quarter, lane, t_base,
-                                    release_cluster_bar, c0, stage, e, k_next);
+    Epi2Staged::body<NC, PRELOAD>(args, Tile2{2 * sc.I + rank, sc.J}, quarter, lane, t_base,
+                                  release_cluster_bar, c0, stage, e, k_next);
   }
 };
 
-template <int EW>
+// Thresholded output (e4m3 tiles) stores little: no staging, and no factors held
+// a tile ahead.  A kernel of its own that has a hit list: as a branch beside the
+// full output's epilogue, and without the assumption, its tests had worse code.
+// GB300, 20,000 SNPs, us per call, branch / by itself / by itself with the
+// assumption: 256 individuals 1145 / 1207 / 1136, 4,096 1863 / 1841 / 1838, 8,192
+// 3322 / 3284 / 3278.
+struct Epi2Filter {
+  using Params = Tally2Args;
+  static constexpr int STAGE_BYTES_PER_WARP = 0;
+  template <int NC>
+  __device__ __forceinline__ static tcp::NoEarly early(const Params &, const TriSchedPair &, bool, int, int, int, int) {
+    return {};
+  }
+  template <int NC, bool PRELOAD = false>
+  __device__ static void tile(const Params &args, const TriSchedPair &sc, int rank, int quarter,
+                              int lane, uint32_t t_base, uint32_t release_cluster_bar, int c0,
+                              float *, tcp::NoEarly, int) {
+    __builtin_assume(args.hits != nullptr);
+    Epi2::body<NC, true, PRELOAD>(args, Tile2{2 * sc.I + rank, sc.J}, quarter, lane, t_base,
+                                  release_cluster_bar, c0);
+  }
+};
+
+template <bool FILTER>
+using Epi2PairOr = std::conditional_t<FILTER, Epi2Filter, Epi2Pair>;
+
+template <int EW, bool FILTER>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * EW, 1)
     k_tally2_tc_pair(const __grid_constant__ CUtensorMap tm, const Tally2Args args,
                      TriSched::Params sp, int nkb) {
-  tcp::persistent_gemm_pair<TriSchedPair, Epi2Pair, EW>(&tm, sp, args, nkb, args.status);
+  tcp::persistent_gemm_pair<TriSchedPair, Epi2PairOr<FILTER>, EW>(&tm, sp, args, nkb, args.status);
 }
 
 // FP4 (e2m1) operands: one accumulator, 8 epilogue warps that load their whole
@@ -805,12 +828,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tcp::SPLIT_THREADS, 
 
 // The pair kernels with the 2-bit codes expanded into count rows in shared
 // memory (tcp::persistent_gemm_pair_packed): no operand matrix in HBM.
-template <int EW>
+template <int EW, bool FILTER>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * EW + 32 * tcp::pk::CW, 1)
     k_tally2_tc_pair_packed(const __grid_constant__ CUtensorMap tmP, const Tally2Args args,
                             TriSched::Params sp, int nkb) {
-  tcp::persistent_gemm_pair_packed<TriSchedPair, Epi2Pair, EW>(&tmP, sp, args, nkb, args.n_v,
-                                                               args.n_f, args.status);
+  tcp::persistent_gemm_pair_packed<TriSchedPair, Epi2PairOr<FILTER>, EW>(
+      &tmP, sp, args, nkb, args.n_v, args.n_f, args.status);
 }
 
 template <int EW>
@@ -1157,10 +1180,12 @@ int launch_tally2_tc_pair(const Tally2Args &a, const uint8_t *op, int64_t rows_p
   const int dev = current_device();
   if (dev < 0) return CCC_ECUDA;
   if (!attr_set[dev]) {
-    if (cudaFuncSetAttribute(k_tally2_tc_pair<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(pair_smem(4))) != cudaSuccess ||
-        cudaFuncSetAttribute(k_tally2_tc_pair<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(pair_smem(8))) != cudaSuccess ||
+    auto allow = [](auto kernel, int ew) {
+      return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  static_cast<int>(pair_smem(ew))) == cudaSuccess;
+    };
+    if (!allow(k_tally2_tc_pair<4, false>, 4) || !allow(k_tally2_tc_pair<8, false>, 8) ||
+        !allow(k_tally2_tc_pair<4, true>, 4) || !allow(k_tally2_tc_pair<8, true>, 8) ||
         !tcp::split_kernel_ready(k_tally2_tc_pair_fp4, pair_smem(tcp::FP4_EW)) ||
         cudaFuncSetAttribute(k_tally2_tc_pair_fp4w, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(rect_smem())) != cudaSuccess)
@@ -1172,7 +1197,8 @@ int launch_tally2_tc_pair(const Tally2Args &a, const uint8_t *op, int64_t rows_p
   if (fp4 && kpad % 256 != 0) return CCC_EINVAL;
   const int64_t row_bytes = fp4 ? kpad / 2 : kpad;
   static int max_clusters[kMaxDevices][4] = {};
-  if (fp4 && a.hits != nullptr) {  // thresholded output: the two-accumulator rect tiles
+  const bool filter = a.hits != nullptr;
+  if (fp4 && filter) {  // thresholded output: the two-accumulator rect tiles
     PairMaps maps;
     if (!make_operand_map(&maps.m[0], op, rows_pad, row_bytes, tcp::BMH) ||
         !make_operand_map(&maps.m[1], op, rows_pad, row_bytes, kRectJ))
@@ -1240,8 +1266,8 @@ int launch_tally2_tc_pair(const Tally2Args &a, const uint8_t *op, int64_t rows_p
     int n = 0;
     const cudaError_t e =
         fp4 ? cudaOccupancyMaxActiveClusters(&n, k_tally2_tc_pair_fp4, &cfg)
-        : ew == 4 ? cudaOccupancyMaxActiveClusters(&n, k_tally2_tc_pair<4>, &cfg)
-                  : cudaOccupancyMaxActiveClusters(&n, k_tally2_tc_pair<8>, &cfg);
+        : ew == 4 ? cudaOccupancyMaxActiveClusters(&n, k_tally2_tc_pair<4, false>, &cfg)
+                  : cudaOccupancyMaxActiveClusters(&n, k_tally2_tc_pair<8, false>, &cfg);
     if (e != cudaSuccess || n < 1) return CCC_ECUDA;
     mc = n < num_sms / 2 ? n : num_sms / 2;
   }
@@ -1249,10 +1275,14 @@ int launch_tally2_tc_pair(const Tally2Args &a, const uint8_t *op, int64_t rows_p
   const int grid = static_cast<int>(2 * clusters);
   if (fp4)
     k_tally2_tc_pair_fp4<<<grid, tcp::SPLIT_THREADS, pair_smem(tcp::FP4_EW), s>>>(tm, a, sp, nkb);
+  else if (ew == 4 && filter)
+    k_tally2_tc_pair<4, true><<<grid, 64 + 32 * 4, pair_smem(4), s>>>(tm, a, sp, nkb);
+  else if (filter)
+    k_tally2_tc_pair<8, true><<<grid, 64 + 32 * 8, pair_smem(8), s>>>(tm, a, sp, nkb);
   else if (ew == 4)
-    k_tally2_tc_pair<4><<<grid, 64 + 32 * 4, pair_smem(4), s>>>(tm, a, sp, nkb);
+    k_tally2_tc_pair<4, false><<<grid, 64 + 32 * 4, pair_smem(4), s>>>(tm, a, sp, nkb);
   else
-    k_tally2_tc_pair<8><<<grid, 64 + 32 * 8, pair_smem(8), s>>>(tm, a, sp, nkb);
+    k_tally2_tc_pair<8, false><<<grid, 64 + 32 * 8, pair_smem(8), s>>>(tm, a, sp, nkb);
   return note_launch();
 }
 
@@ -1382,18 +1412,20 @@ int launch_tally2_tc_pair_packed(const Tally2Args &a, const uint64_t *geno, int6
   const int64_t tiles = tc2_pair_tiles(a.n_v, sp.I0, sp.I1);
   if (tiles == 0) return CCC_OK;
   const int ew = epilogue_warps(nkb);
-  static int cache4[kMaxDevices] = {}, cache8[kMaxDevices] = {};
-  const int mc = ew == 4 ? pair_clusters(k_tally2_tc_pair_packed<4>, 64 + 32 * 4 + CT,
-                                         packed_smem(4), num_sms, cache4)
-                         : pair_clusters(k_tally2_tc_pair_packed<8>, 64 + 32 * 8 + CT,
-                                         packed_smem(8), num_sms, cache8);
-  if (mc < 1) return CCC_ECUDA;
-  const int grid = static_cast<int>(2 * (tiles < mc ? tiles : mc));
-  if (ew == 4)
-    k_tally2_tc_pair_packed<4><<<grid, 64 + 32 * 4 + CT, packed_smem(4), s>>>(tm, a, sp, nkb);
-  else
-    k_tally2_tc_pair_packed<8><<<grid, 64 + 32 * 8 + CT, packed_smem(8), s>>>(tm, a, sp, nkb);
-  return note_launch();
+  static int cache[4][kMaxDevices] = {};
+  auto go = [&](auto kernel, int warps, int(&clusters)[kMaxDevices]) -> int {
+    const int threads = 64 + 32 * warps + CT;
+    const int mc = pair_clusters(kernel, threads, packed_smem(warps), num_sms, clusters);
+    if (mc < 1) return CCC_ECUDA;
+    const int grid = static_cast<int>(2 * (tiles < mc ? tiles : mc));
+    kernel<<<grid, threads, packed_smem(warps), s>>>(tm, a, sp, nkb);
+    return note_launch();
+  };
+  if (a.hits != nullptr)
+    return ew == 4 ? go(k_tally2_tc_pair_packed<4, true>, 4, cache[0])
+                   : go(k_tally2_tc_pair_packed<8, true>, 8, cache[1]);
+  return ew == 4 ? go(k_tally2_tc_pair_packed<4, false>, 4, cache[2])
+                 : go(k_tally2_tc_pair_packed<8, false>, 8, cache[3]);
 }
 
 int launch_tally2_tc_pair_split_packed(const Tally2Args &a, const uint64_t *geno, int64_t ld,
